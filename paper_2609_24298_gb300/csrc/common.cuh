@@ -261,25 +261,6 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
 }
 
-// Rows [0, r) of a basis (fp32, 128 per row, 16-byte aligned) into shared memory with row
-// stride ld floats (a multiple of 4); rows [r, 128) are zeroed.  Every copy is issued before
-// any is waited for.  The caller synchronises the block before reading.
-// issues the copies only; the caller waits with cp_async_wait_all() before reading dst
-__device__ __forceinline__ void stage_basis_issue(const float* W, int r, int ld, float* dst) {
-  for (int idx = threadIdx.x; idx < 128 * 32; idx += blockDim.x) {
-    const int i = idx >> 5, c = idx & 31;
-    float* d = dst + (size_t)i * ld + 4 * c;
-    if (i < r)
-      cp_async16(smem_addr(d), W + (size_t)idx * 4);
-    else
-      *reinterpret_cast<float4*>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-}
-__device__ __forceinline__ void stage_basis(const float* W, int r, int ld, float* dst) {
-  stage_basis_issue(W, r, ld, dst);
-  cp_async_wait_all();
-}
-
 // ---------------------------------------------------------------------------------------
 // parameter block access
 // ---------------------------------------------------------------------------------------

@@ -10,14 +10,14 @@
 namespace cobra {
 
 // ---------------------------------------------------------------------------------------
-// Per-head kernels: the query projection has one CTA of 256 threads per (layer, kv head),
-// looping over the sequences 32 query vectors at a time, with the head's basis staged in
-// shared memory once; the combine has one per (layer, kv head) and run of kCombineVP query
-// vectors.  The workspace's head-group table gives the group of (head, seq).
+// Per-head kernels: the query projection has one CTA of 256 threads per (layer, kv head) and run
+// of sequences, 32 query vectors per pass, with the head's basis staged in shared memory once; the
+// combine has one per (layer, kv head) and run of kCombineVP query vectors.  The workspace's
+// head-group table gives the group of (head, seq).
 // ---------------------------------------------------------------------------------------
 constexpr int kHeadThreads = 256;
 constexpr int kVecPass = 32;  // query vectors (sequences x G) per pass
-constexpr int kWLd = 132;     // padded row stride (floats) of a staged basis: conflict-free row reads
+static_assert(kVecPass + kVecPass / 4 <= kProjVecs, "a pass holds its queries and their sequences' new tokens");
 // row stride of the transposed rank-space averages of a combine pass of VP vectors (odd:
 // the per-channel writes are conflict-free; the reads are broadcasts)
 template <int VP>
@@ -25,11 +25,6 @@ __host__ __device__ constexpr int combine_zld() {
   return VP + 1;
 }
 
-__host__ __device__ constexpr size_t qproj_smem_bytes() {
-  return sizeof(float) * ((size_t)kD * kWLd + (size_t)kVecPass * kD + (size_t)kVecPass * kWLd + kD);
-}
-static_assert(append_smem_bytes() <= qproj_smem_bytes(), "the V-append CTAs use the projection's shared memory");
-static_assert(kWLd == kAppendWLd, "the query projection stages W_K as the append reads it");
 constexpr int kWtChunk = 64;  // chunk weights held in shared memory per vector and round
 constexpr int kCombineVP = 16;  // query vectors per combine CTA (a head's sequences spread over CTAs)
 template <int VP>
@@ -42,97 +37,85 @@ __host__ __device__ constexpr size_t combine_smem_bytes() {
 //   q~_g = (Delta_K / sqrt d) log2(e) W_K^T q_g per query head, scaled by a power of two so
 //   that max |q~| of the group lands in [256, 512), split into fp16 hi + lo and laid out as
 //   the scan's MMA B fragments; Qsum_g = sum over channels of the fed hi + lo values.
-//   With ak.x set, the CTA first appends the new K token of every sequence of its head (a8),
-//   which projects through the same staged W_K.  With av.x set, the grid has a second half of
-//   CTAs (blockIdx.x >= n_qblocks) that append the new V tokens, one (layer, kv head) each, so
-//   that both appends and the projection run in one launch.
+//   With ak.x set, the CTA also appends the new K tokens of its sequences (a8), which project
+//   through the same staged W_K: they are further vectors of the same projection.  With av.x set,
+//   the grid has a second half of CTAs (blockIdx.x >= n_qblocks) that append the new V tokens of
+//   the same runs of sequences, so that both appends and the projection run in one launch.
+//
+//   A latency kernel: a chain of dependent loads (plan, head table, basis), then short phases.
+//   The sequences of a head are spread over n_split CTAs when the heads alone leave SMs idle
+//   (see proj_split), and every phase uses all eight warps whatever the number of vectors.
 // ---------------------------------------------------------------------------------------
 static_assert(kAppendThreads == kHeadThreads, "the V append runs in the query projection's CTAs");
 template <int G>
-__global__ void __launch_bounds__(kHeadThreads) qproj_kernel(DecodeArgs a, CompressArgs ak, CompressArgs av,
-                                                             int n_qblocks) {
+__global__ void __launch_bounds__(kHeadThreads, 2) qproj_kernel(DecodeArgs a, CompressArgs ak, CompressArgs av,
+                                                             int n_qblocks, int n_split, int spb) {
+  extern __shared__ __align__(16) float qsm[];
   grid_dep_launch();
+  const int blk = (int)blockIdx.x % n_qblocks, head = blk / n_split;
+  const int seq0 = (blk % n_split) * spb;
   if ((int)blockIdx.x >= n_qblocks) {
-    extern __shared__ __align__(16) float vsm[];
-    append_block(av, (int)blockIdx.x - n_qblocks, vsm);
+    append_block(av, head, seq0, min(av.n_seqs, seq0 + spb), qsm);
     return;
   }
   constexpr int NTK = Heads<G>::NTK, SPP = kVecPass / G;
-  extern __shared__ __align__(16) float qsm[];
-  float* Ws = qsm;                  // [kD][kWLd]   W_K row i = channel i
-  float* Qs = Ws + kD * kWLd;       // [kVecPass][kD] queries of this pass (fp32); the appended tokens first
-  float* Os = Qs + kVecPass * kD;   // [kVecPass][kWLd] scaled q~ of this pass
-  float* wmu = Os + kVecPass * kWLd;  // [kD] W_K^T mu_K for the append
+  __shared__ float amax_s[kVecPass], up_s[SPP];
+  const ProjSmem sm(qsm);
   const WsHeader* wh = reinterpret_cast<const WsHeader*>(a.ws);
   const WsGroup* groups = reinterpret_cast<const WsGroup*>(a.ws + wh->groups_off);
   const int S = wh->n_seqs;
-  const int* hg = reinterpret_cast<const int*>(a.ws + wh->hg_off) + (size_t)blockIdx.x * S;
+  const int* hg = reinterpret_cast<const int*>(a.ws + wh->hg_off) + (size_t)head * S;
   const WsGroup g0 = groups[hg[0]];
   const HeadEntry hk = head_table(a.block)[g0.k_head];
-  const float* pool = param_pool(a.block);
   const int r = hk.r, layer = g0.layer, kv = g0.kv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int seq1 = min(S, seq0 + spb);
   const float scale = hk.delta * 0.088388347648318440f * 1.4426950408889634f;  // Delta/sqrt(128)*log2(e)
   // the basis is a parameter: its copy overlaps the end of the kernel ahead; the queries, the
   // new tokens, the cache and the q~ blocks of the workspace are touched only after the wait
   const bool append = ak.x != nullptr && r > 0;
-  if (append && tid < (r + 3) / 4) cp_async16(smem_addr(wmu + 4 * tid), pool + hk.wmu_off + 4 * tid);
-  stage_basis_issue(pool + hk.w_off, r, kWLd, Ws);
+  proj_stage_issue(sm, param_pool(a.block), hk);
   grid_dep_wait();
-  if (append) {
-    const AppendNext nx = append_load(ak, layer, kv, warp);
+  const bool wide =
+      ((reinterpret_cast<uintptr_t>(a.q) | (uintptr_t)(2 * a.q_sl) | (uintptr_t)(2 * a.q_ss)) & 15) == 0 &&
+      (!append || append_wide(ak));
+  const __nv_bfloat16* q = a.q + layer * a.q_sl + (long long)(kv * G) * kD;
+  const __nv_bfloat16* x = append ? ak.x + layer * ak.sl + kv * ak.sh : nullptr;
+  for (int s0 = seq0; s0 < seq1; s0 += SPP) {
+    const int ns = min(SPP, seq1 - s0), nq = ns * G, nv = nq + (append ? ns : 0);
+    // vectors: the queries of the pass's sequences, then their new tokens
+    proj_load(
+        nv, wide,
+        [&](int v) {
+          return v < nq ? q + (long long)(s0 + v / G) * a.q_ss + (v % G) * kD : x + (long long)(s0 + v - nq) * ak.ss;
+        },
+        sm.Xs);
+    if (append && tid < ns) sm.pos[tid] = ak.pos[s0 + tid];
     cp_async_wait_all();
+    __syncthreads();  // basis and vectors staged
+    project(sm, nv, r);
     __syncthreads();
-    append_tokens(ak, hk, layer, kv, Ws, wmu, Qs + warp * kD, warp, kHeadThreads / 32, nx);
-  }
-  cp_async_wait_all();
-  for (int s0 = 0; s0 < S; s0 += SPP) {
-    const int ns = min(SPP, S - s0), nv = ns * G;
-    __syncthreads();  // basis staged; the appends and the previous pass are done with Qs and Os
-    // queries are only 2-byte aligned in general: element loads, all issued together
-#pragma unroll 16
-    for (int idx = tid; idx < nv * kD; idx += kHeadThreads) {
-      const int v = idx / kD, d = idx % kD;
-      const __nv_bfloat16* qp = a.q + layer * a.q_sl + (long long)(s0 + v / G) * a.q_ss + (long long)(kv * G + v % G) * kD;
-      Qs[v * kD + d] = __bfloat162float(qp[d]);
-    }
-    __syncthreads();
-    // warp w: vectors 4w..4w+3; lane: channels lane + 32c
-    const int v0 = 4 * warp;
-    if (v0 < nv) {
-      float acc[4][4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[c][v] = 0.f;
-#pragma unroll 4
-      for (int d = 0; d < kD; d += 4) {
-        float4 w[4], q[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) w[c] = *reinterpret_cast<const float4*>(Ws + (lane + 32 * c) * kWLd + d);
-#pragma unroll
-        for (int v = 0; v < 4; ++v) q[v] = *reinterpret_cast<const float4*>(Qs + (v0 + v) * kD + d);
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-#pragma unroll
-          for (int v = 0; v < 4; ++v)
-            acc[c][v] += w[c].x * q[v].x + w[c].y * q[v].y + w[c].z * q[v].z + w[c].w * q[v].w;
+    if (append) append_codes(ak, hk, sm, nq, s0, ns);
+    // per query vector (one warp each): largest |q~|
+    for (int v = warp; v < nq; v += kProjWarps) {
+      float* o = sm.Os + v * kProjLd;
+      float amax = 0.f;
+      for (int i = lane; i < r; i += 32) {
+        const float y = o[i] * scale;
+        o[i] = y;
+        amax = fmaxf(amax, fabsf(y));
       }
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) Os[(v0 + v) * kWLd + lane + 32 * c] = acc[c][v] * scale;
+      for (int m = 16; m; m >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, m));
+      if (lane == 0) amax_s[v] = amax;
     }
     __syncthreads();
-    // per sequence (one warp each): power-of-two scale, hi/lo split, Qsum, B fragments
-    for (int sl = warp; sl < ns; sl += kHeadThreads / 32) {
-      const float* o = Os + sl * G * kWLd;
+    // per query vector: the group's power-of-two scale, Qsum of the hi/lo split
+    for (int v = warp; v < nq; v += kProjWarps) {
+      const int sl = v / G, g = v % G;
       float amax = 0.f;
-      for (int i = lane; i < r; i += 32)
 #pragma unroll
-        for (int g = 0; g < G; ++g) amax = fmaxf(amax, fabsf(o[g * kWLd + i]));
-#pragma unroll
-      for (int m = 16; m; m >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, m));
+      for (int k = 0; k < G; ++k) amax = fmaxf(amax, amax_s[sl * G + k]);
       int e = 0;
       if (amax > 0.f) {
         int ex;
@@ -140,45 +123,52 @@ __global__ void __launch_bounds__(kHeadThreads) qproj_kernel(DecodeArgs a, Compr
         e = 9 - ex;
       }
       const float up = ldexpf(1.f, e);
-      unsigned char* qt = a.ws + wh->qt_off + (size_t)hg[s0 + sl] * wh->qt_stride;
-      float* qhdr = reinterpret_cast<float*>(qt);
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        float sum = 0.f;
-        for (int i = lane; i < r; i += 32) {
-          const float x = o[g * kWLd + i] * up;
-          const __half h = __float2half_rn(x);
-          const __half l = __float2half_rn(x - __half2float(h));
-          sum += __half2float(h) + __half2float(l);
-        }
-#pragma unroll
-        for (int m = 16; m; m >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, m);
-        if (lane == 0) qhdr[g] = sum;
+      const float* o = sm.Os + v * kProjLd;
+      float sum = 0.f;
+      for (int i = lane; i < r; i += 32) {
+        const float y = o[i] * up;
+        const __half h = __float2half_rn(y);
+        const __half l = __float2half_rn(y - __half2float(h));
+        sum += __half2float(h) + __half2float(l);
       }
-      if (lane == 0) qhdr[8] = ldexpf(1.f, -e);
-      // element (k, n) of fragment (kappa, nt) = hi or lo part of q~ of channel 16 kappa + k
-      // for the query head of column n (see Heads)
-      uint2* frag = reinterpret_cast<uint2*>(qt + kQtHeaderBytes);
-      for (int idx = lane; idx < 8 * NTK * 32; idx += 32) {
-        const int fl = idx & 31, nt = (idx >> 5) % NTK, kap = idx / (32 * NTK);
-        const int j = fl & 3, n = fl >> 2;
-        const int g = Heads<G>::col_head(nt, n), lo = Heads<G>::col_lo(nt, n);
-        float e4[4];
-        const int ks[4] = {2 * j, 2 * j + 1, 2 * j + 8, 2 * j + 9};
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int ch = 16 * kap + ks[u];
-          float v = 0.f;
-          if (ch < r) {
-            const float x = o[g * kWLd + ch] * up;
-            const float h = __half2float(__float2half_rn(x));
-            v = lo ? (x - h) : h;
-          }
-          e4[u] = v;
+      for (int m = 16; m; m >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, m);
+      if (lane == 0) {
+        float* qhdr = reinterpret_cast<float*>(a.ws + wh->qt_off + (size_t)hg[s0 + sl] * wh->qt_stride);
+        qhdr[g] = sum;
+        if (g == 0) {
+          qhdr[8] = ldexpf(1.f, -e);
+          up_s[sl] = up;
         }
-        frag[(kap * NTK + nt) * 32 + fl] = make_uint2(pack_f16(e4[0], e4[1]), pack_f16(e4[2], e4[3]));
       }
     }
+    __syncthreads();
+    // element (k, n) of fragment (kappa, nt) = hi or lo part of q~ of channel 16 kappa + k
+    // for the query head of column n (see Heads)
+    for (int idx = tid; idx < ns * 8 * NTK * 32; idx += kHeadThreads) {
+      const int fl = idx & 31, nt = (idx >> 5) % NTK, kap = (idx / (32 * NTK)) & 7, sl = idx / (256 * NTK);
+      const int j = fl & 3, n = fl >> 2;
+      const int g = Heads<G>::col_head(nt, n), lo = Heads<G>::col_lo(nt, n);
+      const float* o = sm.Os + (sl * G + g) * kProjLd;
+      const float up = up_s[sl];
+      float e4[4];
+      const int ks[4] = {2 * j, 2 * j + 1, 2 * j + 8, 2 * j + 9};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int ch = 16 * kap + ks[u];
+        float v = 0.f;
+        if (ch < r) {
+          const float y = o[ch] * up;
+          const float h = __half2float(__float2half_rn(y));
+          v = lo ? (y - h) : h;
+        }
+        e4[u] = v;
+      }
+      unsigned char* qt = a.ws + wh->qt_off + (size_t)hg[s0 + sl] * wh->qt_stride;
+      reinterpret_cast<uint2*>(qt + kQtHeaderBytes)[(kap * NTK + nt) * 32 + fl] =
+          make_uint2(pack_f16(e4[0], e4[1]), pack_f16(e4[2], e4[3]));
+    }
+    __syncthreads();  // Os, pos and the scales are rewritten by the next pass
   }
 }
 

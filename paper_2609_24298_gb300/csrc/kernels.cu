@@ -207,6 +207,22 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, 
 }  // namespace
 
 namespace {
+// How the sequences of each (layer, kv head) are spread over projecting CTAs (append, query
+// projection): n_split CTAs of spb sequences.  Two such CTAs are resident per SM; up to that many
+// of each kind (K and V) run at once, so heads that leave SMs idle are split, down to one sequence
+// per CTA.  Each CTA stages the basis again (32-64 KB from L2), which is why full grids are not.
+// One layer of 8 kv heads, 24 sequences at 3 bpd: a step takes 67 us against 106 with one CTA per
+// head; 8 sequences at 1 bpd 80 against 89; 1 sequence 26 against 28.5.  32 layers of 8 heads run
+// one CTA per head as before (876 us either way).
+struct ProjSplit {
+  int n_split, spb;
+};
+ProjSplit proj_split(long long heads, int n_seqs) {
+  const long long want = std::max(1LL, std::min<long long>(n_seqs, sm_count() / heads));
+  const int spb = (int)((n_seqs + want - 1) / want);
+  return {(n_seqs + spb - 1) / spb, spb};
+}
+
 // validated append arguments for one side
 cobra_status append_args(const void* params, const cobra_compress_desc* d, const void* x, const int* pos,
                          uint8_t* cache, const int* page_table, CompressArgs& a) {
@@ -242,11 +258,12 @@ extern "C" cobra_status cobra_append(const void* params, const cobra_compress_de
   CompressArgs a;
   cobra_status st = append_args(params, d, x, pos, cache, page_table, a);
   if (st != COBRA_OK) return st;
-  const long long grid = (long long)d->n_layers * d->n_kv_heads;  // one CTA per (layer, kv head)
+  const long long heads = (long long)d->n_layers * d->n_kv_heads;
+  const ProjSplit sp = proj_split(heads, d->n_seqs);
   static Granted granted;
-  if (ensure_smem(append_kernel, append_smem_bytes(), granted) != COBRA_OK) return COBRA_ECUDA;
-  if (launch_pdl(append_kernel, (unsigned)grid, kAppendThreads, append_smem_bytes(), (cudaStream_t)stream, a) !=
-      cudaSuccess)
+  if (ensure_smem(append_kernel, proj_smem_bytes(), granted) != COBRA_OK) return COBRA_ECUDA;
+  if (launch_pdl(append_kernel, (unsigned)(heads * sp.n_split), kAppendThreads, proj_smem_bytes(), (cudaStream_t)stream,
+                 a, sp.n_split, sp.spb) != cudaSuccess)
     return COBRA_ECUDA;
   return launch_status();
 }
@@ -260,19 +277,21 @@ cobra_status launch_decode(const DecodeArgs& a, int n_heads, int n_seqs, int n_i
                            bool after_plan_kernel = false, const CompressArgs& ak = CompressArgs{},
                            const CompressArgs& av = CompressArgs{}) {
   static Granted qproj_granted, combine_granted;
-  if (ensure_smem(qproj_kernel<G>, qproj_smem_bytes(), qproj_granted) != COBRA_OK ||
+  if (ensure_smem(qproj_kernel<G>, proj_smem_bytes(), qproj_granted) != COBRA_OK ||
       ensure_smem(combine_kernel<G, kCombineVP>, combine_smem_bytes<kCombineVP>(), combine_granted) != COBRA_OK)
     return COBRA_ECUDA;
   if (stages & kQproj) {
     // the query projection reads the plan before its wait; right after the plan kernel it is
     // launched in plain stream order
-    // with a V append, its CTAs follow the projection's (one per (layer, kv head))
-    const unsigned grid = (unsigned)n_heads * (av.x ? 2u : 1u);
+    // with a V append, its CTAs follow the projection's (as many, over the same sequences)
+    const ProjSplit sp = proj_split(n_heads, n_seqs);
+    const int n_qblocks = n_heads * sp.n_split;
+    const unsigned grid = (unsigned)n_qblocks * (av.x ? 2u : 1u);
     if (after_plan_kernel) {
-      qproj_kernel<G><<<grid, kHeadThreads, qproj_smem_bytes(), s>>>(a, ak, av, n_heads);
+      qproj_kernel<G><<<grid, kHeadThreads, proj_smem_bytes(), s>>>(a, ak, av, n_qblocks, sp.n_split, sp.spb);
       if (cudaGetLastError() != cudaSuccess) return COBRA_ECUDA;
-    } else if (launch_pdl(qproj_kernel<G>, grid, kHeadThreads, qproj_smem_bytes(), s, a, ak, av, n_heads) !=
-               cudaSuccess) {
+    } else if (launch_pdl(qproj_kernel<G>, grid, kHeadThreads, proj_smem_bytes(), s, a, ak, av, n_qblocks, sp.n_split,
+                          sp.spb) != cudaSuccess) {
       return COBRA_ECUDA;
     }
   }
