@@ -12,25 +12,13 @@ namespace cobra {
 // ---------------------------------------------------------------------------------------
 // Per-head kernels: the query projection has one CTA of 256 threads per (layer, kv head) and run
 // of sequences, 32 query vectors per pass, with the head's basis staged in shared memory once; the
-// combine has one per (layer, kv head) and run of kCombineVP query vectors.  The workspace's
-// head-group table gives the group of (head, seq).
+// combine has one per (layer, kv head, sequence).  The workspace's head-group table gives the group
+// of (head, seq).
 // ---------------------------------------------------------------------------------------
 constexpr int kHeadThreads = 256;
 constexpr int kVecPass = 32;  // query vectors (sequences x G) per pass
 static_assert(kVecPass + kVecPass / 4 <= kProjVecs, "a pass holds its queries and their sequences' new tokens");
-// row stride of the transposed rank-space averages of a combine pass of VP vectors (odd:
-// the per-channel writes are conflict-free; the reads are broadcasts)
-template <int VP>
-__host__ __device__ constexpr int combine_zld() {
-  return VP + 1;
-}
-
 constexpr int kWtChunk = 64;  // chunk weights held in shared memory per vector and round
-constexpr int kCombineVP = 16;  // query vectors per combine CTA (a head's sequences spread over CTAs)
-template <int VP>
-__host__ __device__ constexpr size_t combine_smem_bytes() {
-  return sizeof(float) * ((size_t)kD * combine_zld<VP>() + kD + (size_t)VP * kWtChunk);
-}
 
 // ---------------------------------------------------------------------------------------
 // a4: query projection
@@ -176,244 +164,190 @@ __global__ void __launch_bounds__(kHeadThreads, 2) qproj_kernel(DecodeArgs a, Co
 // a7: combine chunks + back-projection
 //   per query head: m* = max over chunks, l* = sum 2^(m - m*) l, zbar = Delta_V (sum 2^(m - m*)
 //   acc / l* - 2^{b-1} + 1/2), o = mu_V + W_V zbar (zeros for an empty sequence).
+//
+// One CTA of 256 threads per (layer, kv head, sequence).  The kernel is a chain of memory round
+// trips (chunk maxima, chunk sums, the rows of W_V), so every phase spreads its loads over all
+// threads and issues them together; a head's W_V is read again for each sequence (from L2).
+// Against one CTA per head and run of 16 query vectors, a step over 1 layer x 8 kv heads takes
+// 23 us for 25.9 (1 x 2048 tokens), 50 for 67 (24 ragged sequences at 3 bpd) and 63 for 80
+// (8 x 32768); over all 32 layers it takes the same 876 us.
 // ---------------------------------------------------------------------------------------
-// One CTA per (layer, kv head) and run of VP / G sequences (VP query vectors).
-template <int G, int VP>
-__global__ void __launch_bounds__(kHeadThreads, 4) combine_kernel(DecodeArgs a) {
-  constexpr int SPP = VP / G > 0 ? VP / G : 1;
-  static_assert(VP % 8 == 0, "combine pass width");
-  constexpr int kZLd = combine_zld<VP>();
-  extern __shared__ __align__(16) float csm[];
-  float* Zs = csm;                  // [kD][kZLd]   zbar of this pass, [channel][vector]
-  float* mus = Zs + kD * kZLd;      // [kD]         mu_V
-  float* wts = mus + kD;            // [VP][kWtChunk] normalised chunk weights
-  __shared__ float vinfo_m[VP], vinfo_inv_l[VP];
-  __shared__ int vinfo_first[VP], vinfo_n[VP], vinfo_g[VP], vinfo_seq[VP];
+template <int G>
+__global__ void __launch_bounds__(kHeadThreads, 3) combine_kernel(DecodeArgs a) {
+  __shared__ float wts[G][kWtChunk];          // weights 2^(m_k - m*) / l* of a round of chunks
+  __shared__ float m_s[G], inv_l_s[G];
+  __shared__ __align__(16) float red[kHeadThreads * 4];  // partial chunk sums, then zbar [channel][G]
   const WsHeader* wh = reinterpret_cast<const WsHeader*>(a.ws);
   const WsGroup* groups = reinterpret_cast<const WsGroup*>(a.ws + wh->groups_off);
   const float* parts = reinterpret_cast<const float*>(a.ws + wh->part_off);
-  const int S = wh->n_seqs;
-  const int nchunks = (S + SPP - 1) / SPP;
-  const int chunk = blockIdx.x % nchunks;
-  const int* hg = reinterpret_cast<const int*>(a.ws + wh->hg_off) + (size_t)(blockIdx.x / nchunks) * S;
-  const WsGroup g0 = groups[hg[0]];
-  const HeadEntry hv = head_table(a.block)[g0.v_head];
+  const int S = wh->n_seqs, pstride = wh->part_stride, gstride = wh->g_stride;
+  const WsGroup gr = groups[reinterpret_cast<const int*>(a.ws + wh->hg_off)[blockIdx.x]];
+  const HeadEntry hv = head_table(a.block)[gr.v_head];
   const float* pool = param_pool(a.block);
-  const int rv = hv.r, layer = g0.layer, kv = g0.kv;
-  const int tid = threadIdx.x;
-  const float cen = rv > 0 ? (float)(1 << (hv.b - 1)) - 0.5f : 0.f;
-  if (tid < kD) mus[tid] = pool[hv.mu_off + tid];
-  // the rows of W_V are read through L1 in the back-projection (every warp reads the same rows);
-  // they are pulled into L2 here, while the scan ahead of this kernel is still finishing
-  const float4* W4 = reinterpret_cast<const float4*>(pool + hv.w_off);
-  for (int idx = tid; idx < rv * (kD / 32); idx += kHeadThreads) prefetch_l2(pool + hv.w_off + 32 * idx);
-  // the plan side of every vector: its group's chunks and query head
-  const int s0 = chunk * SPP;
-  const int ns = min(SPP, S - s0), nv = ns * G;
-  if (tid < nv) {
-    const WsGroup gr = groups[hg[s0 + tid / G]];
-    vinfo_first[tid] = gr.first_item;
-    vinfo_n[tid] = gr.n_items;
-    vinfo_g[tid] = tid % G;
-    vinfo_seq[tid] = gr.seq;
-  }
+  const int rv = hv.r, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const float* W = pool + hv.w_off;
+  // W_V is pulled into L2 here, while the scan ahead of this kernel is still finishing (the first
+  // sequence's CTA of a head does it for all)
+  if (blockIdx.x % S == 0)
+    for (int idx = tid; idx < rv * (kD / 32); idx += kHeadThreads) prefetch_l2(W + 32 * idx);
+  const int d0 = 16 * warp + 4 * (lane & 3);  // dims of the back-projection: d0 .. d0 + 3
+  const float4 mu4 = *reinterpret_cast<const float4*>(pool + hv.mu_off + d0);
   // the appends of the next step may start their parameter staging meanwhile
   grid_dep_launch();
   // everything above is independent of the scan; its partials are read only from here on
   grid_dep_wait();
+  const int n = a.seq_lens[gr.seq] > 0 ? gr.n_items : 0;
+  const float* part = parts + (size_t)gr.first_item * pstride;
+  // (1) warp g: m* and l* of query head g, lanes over chunks, merged online (a chunk with no tokens
+  //     has m = -inf and no value entries; its weight is zero).  The m of the first kWtChunk chunks
+  //     stay in shared memory and become the weights of the first round of (2).
+  if (warp < G) {
+    const float* pg = part + warp * gstride;
+    float M = -INFINITY, Ls = 0.f;
+    for (int k = lane; k < n; k += 32) {
+      const float mk = pg[(size_t)k * pstride], lk = pg[(size_t)k * pstride + 1];
+      if (k < kWtChunk) wts[warp][k] = mk;
+      if (mk == -INFINITY) continue;
+      const float mn = fmaxf(M, mk);
+      Ls = Ls * exp2f(M - mn) + lk * exp2f(mk - mn);
+      M = mn;
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      const float mo = __shfl_xor_sync(0xffffffffu, M, o), lo = __shfl_xor_sync(0xffffffffu, Ls, o);
+      const float mn = fmaxf(M, mo);
+      if (mn != -INFINITY) {
+        Ls = Ls * exp2f(M - mn) + lo * exp2f(mo - mn);
+        M = mn;
+      }
+    }
+    const float inv_l = n > 0 ? 1.f / Ls : 0.f;
+    if (lane == 0) {
+      m_s[warp] = M;
+      inv_l_s[warp] = inv_l;
+    }
+    // the same lane wrote wts[..][k] above for k < n
+    for (int k = lane; k < min(n, kWtChunk); k += 32) {
+      const float mk = wts[warp][k];
+      wts[warp][k] = mk != -INFINITY ? exp2f(mk - M) * inv_l : 0.f;
+    }
+  }
+  __syncthreads();
+  // (2) weighted chunk sums: thread (channel quad cq, query head g, chunk share p) of rw = r_V
+  //     rounded up to 32, 64 or 128 channels sums 16-byte entries of chunks p, p + np, ..., eight
+  //     loads in flight; the shares are added through shared memory.
+  const int rw = rv <= 32 ? 32 : rv <= 64 ? 64 : kD;
+  const int nq = rw / 4, np = kHeadThreads / (nq * G);  // np >= 1 (G = 8, rw = 128)
   {
-    __syncthreads();  // mu_V and the vector table staged
-    // (1) per vector (warp w: vectors w, w + 8, ...): m* = max over the chunks and
-    //     l* = sum 2^(m - m*) l, lanes over chunks, merged online (a chunk with no tokens has
-    //     m = -inf and no value entries; its weight is zero).  The vectors' loads are issued
-    //     together; the lanes keep the m of the first kWtChunk chunks and turn them into the
-    //     weights 2^(m - m*) / l* of the first round of (2).
-    const int warp = tid >> 5, lane = tid & 31;
-    constexpr int NU = VP / (kHeadThreads / 32);
-    {
-      const float* pg0[NU];
-      int ni[NU];
-      float M[NU], Lsum[NU];
-      int kmax = 0;
-#pragma unroll
-      for (int u = 0; u < NU; ++u) {
-        const int v = warp + 8 * u;
-        ni[u] = (v < nv && a.seq_lens[vinfo_seq[v]] > 0) ? vinfo_n[v] : 0;
-        pg0[u] = parts + (v < nv ? (size_t)vinfo_first[v] * wh->part_stride + (v % G) * wh->g_stride : 0);
-        M[u] = -INFINITY;
-        Lsum[u] = 0.f;
-        kmax = max(kmax, ni[u]);
-      }
-      for (int k = lane; k < kmax; k += 32) {
-        float mk[NU], lk[NU];
-#pragma unroll
-        for (int u = 0; u < NU; ++u) {
-          const bool ok = k < ni[u];
-          mk[u] = ok ? pg0[u][(size_t)k * wh->part_stride] : -INFINITY;
-          lk[u] = ok ? pg0[u][(size_t)k * wh->part_stride + 1] : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < NU; ++u) {
-          if (k < kWtChunk && warp + 8 * u < nv) wts[(warp + 8 * u) * kWtChunk + k] = mk[u];
-          if (mk[u] == -INFINITY) continue;
-          const float mn = fmaxf(M[u], mk[u]);
-          Lsum[u] = Lsum[u] * exp2f(M[u] - mn) + lk[u] * exp2f(mk[u] - mn);
-          M[u] = mn;
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < NU; ++u) {
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-          const float mo = __shfl_xor_sync(0xffffffffu, M[u], o), lo = __shfl_xor_sync(0xffffffffu, Lsum[u], o);
-          const float mn = fmaxf(M[u], mo);
-          if (mn != -INFINITY) {
-            Lsum[u] = Lsum[u] * exp2f(M[u] - mn) + lo * exp2f(mo - mn);
-            M[u] = mn;
+    const int cq = tid % nq, g = (tid / nq) % G, p = tid / (nq * G);
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k0 = 0; k0 < n; k0 += kWtChunk) {
+      if (k0 > 0) {  // later rounds: one weight per thread into shared memory
+        __syncthreads();
+        for (int idx = tid; idx < G * kWtChunk; idx += kHeadThreads) {
+          const int v = idx / kWtChunk, k = k0 + idx % kWtChunk;
+          float w = 0.f;
+          if (k < n) {
+            const float mk = part[(size_t)k * pstride + v * gstride];
+            if (mk != -INFINITY) w = exp2f(mk - m_s[v]) * inv_l_s[v];
           }
+          wts[v][idx % kWtChunk] = w;
         }
-        const int v = warp + 8 * u;
-        if (v >= nv) continue;
-        const float inv_l = ni[u] > 0 ? 1.f / Lsum[u] : 0.f;
-        if (lane == 0) {
-          vinfo_first[v] = ni[u] > 0 ? vinfo_first[v] : -1;
-          vinfo_n[v] = ni[u];
-          vinfo_m[v] = M[u];
-          vinfo_inv_l[v] = inv_l;
+        __syncthreads();
+      }
+      if (4 * cq >= rv) continue;
+      // the partial's channels start 4 floats in and every stride is a multiple of 4 floats
+      const float4* px = reinterpret_cast<const float4*>(part + (size_t)k0 * pstride + g * gstride + 4 + 4 * cq);
+      const int kr = min(kWtChunk, n - k0);
+      for (int kb = p; kb < kr; kb += 8 * np) {
+        float4 x[8];
+        float w[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int k = kb + u * np;
+          w[u] = k < kr ? wts[g][k] : 0.f;
+          // an empty chunk's value entries were never written
+          x[u] = w[u] != 0.f ? px[(size_t)k * (pstride / 4)] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        // the same lane wrote wts[v][k] above for k < kmax
-        for (int k = lane; k < kWtChunk; k += 32) {
-          const float mk = k < ni[u] ? wts[v * kWtChunk + k] : -INFINITY;
-          wts[v * kWtChunk + k] = mk != -INFINITY ? exp2f(mk - M[u]) * inv_l : 0.f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          acc.x += w[u] * x[u].x;
+          acc.y += w[u] * x[u].y;
+          acc.z += w[u] * x[u].z;
+          acc.w += w[u] * x[u].w;
         }
       }
+    }
+    *reinterpret_cast<float4*>(red + 4 * tid) = acc;
+  }
+  __syncthreads();
+  // zbar = Delta (sum_k w_k acc_k - 2^{b-1} + 1/2), written back as [channel][G]
+  {
+    const float cen = rv > 0 ? (float)(1 << (hv.b - 1)) - 0.5f : 0.f;
+    float z[G / 2];  // at most G rw / 256 <= G / 2 values per thread
+#pragma unroll
+    for (int u = 0; u < G / 2; ++u) {
+      const int idx = tid + u * kHeadThreads;  // g rw + channel
+      float sum = 0.f;
+      if (idx < G * rw)
+        for (int p = 0; p < np; ++p) sum += red[p * G * rw + idx];
+      z[u] = n > 0 ? hv.delta * (sum - cen) : 0.f;
     }
     __syncthreads();
-    // (2) zbar[v][i] = Delta (sum_k w_k acc_k[i] - 2^{b-1} + 1/2) with w_k = 2^(m_k - m*) / l*.
-    //     Rounds of kWtChunk chunks (the first round's weights come from (1); later rounds
-    //     compute them one (vector, chunk) per thread into shared memory).  Thread (channel
-    //     quad cq, slot) of rw = r_V rounded up to 32, 64 or 128 channels holds channels
-    //     4 cq .. 4 cq + 3 of the vectors slot, slot + ns, ... (ns = 256 / (rw / 4) slots) and
-    //     sums over the chunks in blocks of KB, the 16-byte loads of all its vectors' KB chunks
-    //     issued before any is used.
-    {
-      constexpr int VPT = (VP + 7) / 8;  // vectors per thread at most (ns >= 8)
-      constexpr int KB = VPT >= 4 ? 4 : 8;  // chunks per block: VPT x KB 16-byte loads in flight
-      const int rw = rv <= 32 ? 32 : rv <= 64 ? 64 : kD;
-      const int nq = rw / 4, ns = kHeadThreads / nq;
-      const int cq = tid % nq, slot = tid / nq;
-      const int pstride = wh->part_stride;
-      int kmax = 0;
-      for (int v = 0; v < nv; ++v) kmax = max(kmax, vinfo_n[v]);
-      float4 acc[VPT];
 #pragma unroll
-      for (int q = 0; q < VPT; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int k0 = 0; k0 < kmax; k0 += kWtChunk) {
-        if (k0 > 0) {
-          __syncthreads();  // the previous round's weights are consumed
-          for (int idx = tid; idx < nv * kWtChunk; idx += kHeadThreads) {
-            const int v = idx / kWtChunk, k = k0 + idx % kWtChunk;
-            float w = 0.f;
-            if (k < vinfo_n[v]) {
-              const float mk = parts[(size_t)(vinfo_first[v] + k) * pstride + vinfo_g[v] * wh->g_stride];
-              if (mk != -INFINITY) w = exp2f(mk - vinfo_m[v]) * vinfo_inv_l[v];
-            }
-            wts[idx] = w;
-          }
-          __syncthreads();
-        }
-        if (4 * cq >= rv) continue;
-        const int kr = min(kWtChunk, kmax - k0);
-        for (int kb = 0; kb < kr; kb += KB) {
-          float4 x[VPT][KB];
+    for (int u = 0; u < G / 2; ++u) {
+      const int idx = tid + u * kHeadThreads;
+      if (idx < G * rw) red[(idx % rw) * G + idx / rw] = z[u];
+    }
+  }
+  __syncthreads();
+  // (3) o = mu_V + W_V zbar: a warp has 16 dims, its lanes 4 dims x every eighth row of W_V (eight
+  //     16-byte loads in flight); the eight row shares are added by halving exchanges, after which
+  //     a lane holds G / 2 consecutive outputs.
+  float o[4 * G];
 #pragma unroll
-          for (int q = 0; q < VPT; ++q) {
-            const int v = slot + ns * q;
-            const int n = v < nv ? vinfo_n[v] - k0 : 0;
-            // the partial's channels start 4 floats in and every stride is a multiple of 4 floats
-            const float4* px = reinterpret_cast<const float4*>(
-                parts + (size_t)max(vinfo_first[v < nv ? v : 0], 0) * pstride + (size_t)k0 * pstride +
-                (v < nv ? vinfo_g[v] : 0) * wh->g_stride + 4 + 4 * cq);
+  for (int k = 0; k < 4 * G; ++k) o[k] = 0.f;
+  const int sl = lane >> 2;
+  const float4* W4 = reinterpret_cast<const float4*>(W + d0);
+  for (int i0 = sl; i0 < rv; i0 += 64) {
+    float4 w[8];
 #pragma unroll
-            for (int kk = 0; kk < KB; ++kk)
-              x[q][kk] = (kb + kk < n) ? px[(size_t)(kb + kk) * (pstride / 4)] : make_float4(0.f, 0.f, 0.f, 0.f);
-          }
+    for (int u = 0; u < 8; ++u)
+      w[u] = i0 + 8 * u < rv ? __ldg(W4 + (i0 + 8 * u) * (kD / 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-          for (int q = 0; q < VPT; ++q) {
-            const int v = slot + ns * q;
-            if (v >= nv) break;
-            const float* wv = wts + v * kWtChunk + kb;
+    for (int u = 0; u < 8; ++u) {
+      // rows past r_V have w = 0; their zbar is finite (zeros, or within rw <= 128 rows)
+      const float* zr = red + (i0 + 8 * u < rv ? i0 + 8 * u : 0) * G;
 #pragma unroll
-            for (int kk = 0; kk < KB; ++kk) {
-              const float w = (kb + kk < kWtChunk) ? wv[kk] : 0.f;
-              if (w != 0.f) {  // an empty chunk's value entries were never written
-                acc[q].x += w * x[q][kk].x;
-                acc[q].y += w * x[q][kk].y;
-                acc[q].z += w * x[q][kk].z;
-                acc[q].w += w * x[q][kk].w;
-              }
-            }
-          }
-        }
-      }
-      if (4 * cq < rv) {
-#pragma unroll
-        for (int q = 0; q < VPT; ++q) {
-          const int v = slot + ns * q;
-          if (v >= nv) break;
-          const bool live = vinfo_first[v] >= 0;
-          const float a4[4] = {acc[q].x, acc[q].y, acc[q].z, acc[q].w};
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-            if (4 * cq + c < rv) Zs[(4 * cq + c) * kZLd + v] = live ? hv.delta * (a4[c] - cen) : 0.f;
-        }
+      for (int g = 0; g < G; ++g) {
+        const float zz = zr[g];
+        o[4 * g + 0] += w[u].x * zz;
+        o[4 * g + 1] += w[u].y * zz;
+        o[4 * g + 2] += w[u].z * zz;
+        o[4 * g + 3] += w[u].w * zz;
       }
     }
-    __syncthreads();
-    // thread: dims 4 (tid % 32) .. +3 for vectors VPW (tid / 32) .. +VPW-1
-    constexpr int VPW = VP / (kHeadThreads / 32);
-    const int d0 = 4 * (tid & 31), v0 = VPW * (tid >> 5);
-    if (v0 < nv) {
-      const float4 m4 = *reinterpret_cast<const float4*>(mus + d0);
-      float4 o[VPW];
+  }
 #pragma unroll
-      for (int v = 0; v < VPW; ++v) o[v] = m4;
-      auto accum = [&](const float4& w, int i) {
-        float zz[VPW];
+  for (int st = 0; st < 3; ++st) {
+    const int half = (4 * G) >> (st + 1), bit = 16 >> st;
+    const bool up = lane & bit;
 #pragma unroll
-        for (int v = 0; v < VPW; ++v) zz[v] = Zs[i * kZLd + v0 + v];
-#pragma unroll
-        for (int v = 0; v < VPW; ++v) {
-          o[v].x += w.x * zz[v];
-          o[v].y += w.y * zz[v];
-          o[v].z += w.z * zz[v];
-          o[v].w += w.w * zz[v];
-        }
-      };
-      // rows in blocks of 8 whose loads are all issued before the first is used
-      int i = 0;
-      for (; i + 8 <= rv; i += 8) {
-        float4 w[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) w[u] = __ldg(W4 + (i + u) * (kD / 4) + (d0 >> 2));
-#pragma unroll
-        for (int u = 0; u < 8; ++u) accum(w[u], i + u);
-      }
-      for (; i < rv; ++i) accum(__ldg(W4 + i * (kD / 4) + (d0 >> 2)), i);
-#pragma unroll
-      for (int v = 0; v < VPW; ++v) {
-        const int vv = v0 + v;
-        if (vv >= nv) break;
-        const int seq = s0 + vv / G, g = vv % G;
-        const bool empty = vinfo_first[vv] < 0;  // a sequence without tokens
-        float* out = a.out + layer * a.o_sl + seq * a.o_ss + (long long)(kv * G + g) * kD + d0;
-        const float4 y = empty ? make_float4(0.f, 0.f, 0.f, 0.f) : o[v];
-        out[0] = y.x;  // the output is only 4-byte aligned in general
-        out[1] = y.y;
-        out[2] = y.z;
-        out[3] = y.w;
+    for (int k = 0; k < (4 * G) >> 1; ++k) {
+      if (k < half) {
+        const float send = up ? o[k] : o[half + k], keep = up ? o[half + k] : o[k];
+        o[k] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
       }
     }
+  }
+  // lane share sl holds outputs [sl G / 2, (sl + 1) G / 2) of the 4 G (query head, dim) values
+  const float mu_a[4] = {mu4.x, mu4.y, mu4.z, mu4.w};
+#pragma unroll
+  for (int k = 0; k < G / 2; ++k) {
+    const int e = sl * (G / 2) + k, g = e >> 2, c = e & 3;
+    const float mu = (G == 8) ? mu_a[k & 3] : ((sl & 1) ? mu_a[2 + k] : mu_a[k]);
+    // the output is only 4-byte aligned in general
+    a.out[gr.layer * a.o_sl + gr.seq * a.o_ss + (long long)(gr.kv * G + g) * kD + d0 + c] = n > 0 ? mu + o[k] : 0.f;
   }
 }
 

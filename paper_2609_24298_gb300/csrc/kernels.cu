@@ -276,10 +276,8 @@ template <int G>
 cobra_status launch_decode(const DecodeArgs& a, int n_heads, int n_seqs, int n_items, int stages, cudaStream_t s,
                            bool after_plan_kernel = false, const CompressArgs& ak = CompressArgs{},
                            const CompressArgs& av = CompressArgs{}) {
-  static Granted qproj_granted, combine_granted;
-  if (ensure_smem(qproj_kernel<G>, proj_smem_bytes(), qproj_granted) != COBRA_OK ||
-      ensure_smem(combine_kernel<G, kCombineVP>, combine_smem_bytes<kCombineVP>(), combine_granted) != COBRA_OK)
-    return COBRA_ECUDA;
+  static Granted qproj_granted;
+  if (ensure_smem(qproj_kernel<G>, proj_smem_bytes(), qproj_granted) != COBRA_OK) return COBRA_ECUDA;
   if (stages & kQproj) {
     // the query projection reads the plan before its wait; right after the plan kernel it is
     // launched in plain stream order
@@ -310,14 +308,11 @@ cobra_status launch_decode(const DecodeArgs& a, int n_heads, int n_seqs, int n_i
     if (launch_pdl(decode_kernel<G>, (unsigned)grid, kDecodeWarps * 32, smem, s, a) != cudaSuccess) return COBRA_ECUDA;
   }
   if (stages & kCombine) {
-    // one CTA per (layer, kv head) and run of kCombineVP / G sequences
-    constexpr int spp = kCombineVP / G > 0 ? kCombineVP / G : 1;
-    const long long grid = (long long)n_heads * ((n_seqs + spp - 1) / spp);
+    // one CTA per (layer, kv head, sequence); its prologue (the plan, the L2 prefetch of W_V)
+    // overlaps the scan's tail
+    const long long grid = (long long)n_heads * n_seqs;
     if (grid > 0x7fffffffLL) return COBRA_EINVAL;
-    // its prologue (mu_V, the L2 prefetch of W_V) overlaps the scan's tail
-    if (launch_pdl(combine_kernel<G, kCombineVP>, (unsigned)grid, kHeadThreads, combine_smem_bytes<kCombineVP>(), s,
-                   a) != cudaSuccess)
-      return COBRA_ECUDA;
+    if (launch_pdl(combine_kernel<G>, (unsigned)grid, kHeadThreads, 0, s, a) != cudaSuccess) return COBRA_ECUDA;
   }
   return COBRA_OK;
 }
