@@ -375,8 +375,8 @@ cobra_status cobra_rope_table(double theta, int max_pos, float* table, size_t ta
  * cobra_rope_table.  A query position or sequence length outside the table, or a head whose
  * code rows do not fit the kernel's staging, is reported through the device status word
  * (cobra_check returns COBRA_EINVAL) and computed with clamped angles or skipped.  The
- * reconstructed keys must stay below 2^14 Delta_K (|mu_K| small against Delta_K 2^15).
- * Three launches: query rotation, scan, combine + back-projection; nothing is synchronised. */
+ * means must stay below 65504 Delta_K (they enter the rebuilt keys as f16 limbs of mu_K / Delta_K).
+ * Two launches: scan, combine + back-projection; nothing is synchronised. */
 cobra_status cobra_decode_rope_attn(const void* params, const cobra_decode_desc* desc, const cobra_decode_info* info,
                                     const void* q, const int* q_pos, const float* rope_table, int max_pos,
                                     const uint8_t* cache, const int* seq_lens, const int* page_table, float* out,

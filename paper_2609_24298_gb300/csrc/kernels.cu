@@ -464,30 +464,36 @@ int smem_optin() {
 }
 
 template <int G>
-cobra_status launch_rope(const DecodeArgs& a, const RopeArgs& ra0, int n_heads, int n_seqs, int n_groups,
-                         int n_items, int max_row_bytes, int max_stage_bytes, cudaStream_t s) {
+cobra_status launch_rope(const DecodeArgs& a, const RopeArgs& ra0, int n_heads, int n_seqs, int n_items,
+                         int max_row_bytes, int max_stage_bytes, cudaStream_t s) {
   RopeArgs ra = ra0;
   // a stage holds the channel tiles of a K row and a V row: the plan's largest, else a bound
-  // from the largest row (at most 1792 bytes of tiles past a K row); the two stages of a warp
-  // also hold its partial for the merge
+  // from the largest row (at most 1792 bytes of tiles past a K row)
   const size_t rowb = (size_t)std::max(max_row_bytes, 16);
   const size_t need = max_stage_bytes > 0 ? (size_t)max_stage_bytes
                                           : align_up(rowb + 1792, 128) + align_up(rowb, 128);
-  const size_t stage = std::max<size_t>(align_up(need, 128), 2560);
+  const size_t stage = std::max<size_t>(align_up(need, 128), 128);
   ra.stage_bytes = (int)stage;
-  const size_t fixed = rope_fixed_bytes<G>(), per_warp = rope_warp_bytes<G>((int)stage);
-  const long long room = (long long)smem_optin() - 1024 - (long long)fixed;
-  const int nw = (int)std::min<long long>(kRopeMaxWarps, room > 0 ? room / (long long)per_warp : 0);
-  if (nw < 1) return COBRA_EINVAL;  // code rows too large for the staging
-  const size_t smem = fixed + (size_t)nw * per_warp;
+  // two warpgroups with two stages each where they fit (up to about 4 bits per dimension on both
+  // sides), else with one stage, else one warpgroup
+  const size_t fixed = rope_fixed_bytes<G>();
+  const long long room = (long long)smem_optin() - (long long)fixed;
+  const long long fit = room > 0 ? room / (long long)stage : 0;
+  if (fit < 1) return COBRA_EINVAL;  // code rows too large for the staging
+  const int nwg = fit >= 2 ? 2 : 1;
+  ra.n_stage = fit >= 2 * nwg ? 2 : 1;
+  const size_t smem = fixed + (size_t)(nwg * ra.n_stage) * stage;
   static Granted granted;
   if (ensure_smem(rope_scan_kernel<G>, smem, granted) != COBRA_OK) return COBRA_ECUDA;
-  if (launch_pdl(rope_qprep_kernel<G>, (unsigned)n_heads, kHeadThreads, 0, s, a, ra) != cudaSuccess)
+  // chunks taken at a time: W_K is staged again for each take, so a call that does not fill the GPU
+  // four times over is dealt out in one take per CTA, a larger one in four or more (the chunks
+  // shrink towards the end of the plan).  The work counter is 0 here (the plan writes it so, every
+  // scan resets it).
+  const int sms = sm_count();
+  ra.batch = n_items <= 4 * sms ? (n_items + sms - 1) / sms : (n_items + 4 * sms - 1) / (4 * sms);
+  const int grid = std::max(1, std::min((n_items + ra.batch - 1) / ra.batch, sms));
+  if (launch_pdl(rope_scan_kernel<G>, (unsigned)grid, (unsigned)(160 * nwg), smem, s, a, ra) != cudaSuccess)
     return COBRA_ECUDA;
-  // one CTA per SM over the groups; the work counter is 0 here (the plan writes it so, every
-  // scan resets it)
-  const int grid = std::max(1, std::min(n_groups, sm_count()));
-  if (launch_pdl(rope_scan_kernel<G>, (unsigned)grid, nw * 32, smem, s, a, ra) != cudaSuccess) return COBRA_ECUDA;
   return launch_decode<G>(a, n_heads, n_seqs, n_items, kCombine, s);
 }
 
@@ -533,10 +539,8 @@ extern "C" cobra_status cobra_decode_rope_attn(const void* params, const cobra_d
   const int n_heads = d->n_layers * d->n_kv_heads;
   cudaStream_t s = (cudaStream_t)stream;
   cobra_status r = d->group == 4
-                       ? launch_rope<4>(a, ra, n_heads, d->n_seqs, info->n_groups, info->n_items,
-                                        info->max_row_bytes, info->max_stage_bytes, s)
-                       : launch_rope<8>(a, ra, n_heads, d->n_seqs, info->n_groups, info->n_items,
-                                        info->max_row_bytes, info->max_stage_bytes, s);
+                       ? launch_rope<4>(a, ra, n_heads, d->n_seqs, info->n_items, info->max_row_bytes, info->max_stage_bytes, s)
+                       : launch_rope<8>(a, ra, n_heads, d->n_seqs, info->n_items, info->max_row_bytes, info->max_stage_bytes, s);
   return r != COBRA_OK ? r : launch_status();
 }
 
