@@ -787,9 +787,12 @@ extern "C" cobra_status cobra_measure_distortion(int n_heads, int n_tok, const f
     if (cobra_loading_factor(b_list[j], &a.L[j]) != COBRA_OK) return COBRA_EINVAL;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  coords_kernel<<<dim3((unsigned)((n_tok + kCoordTok - 1) / kCoordTok), (unsigned)n_heads), 256, 0, s>>>(a);
+  static Granted granted;
+  if (ensure_smem(coords_kernel, proj_smem_bytes(), granted) != COBRA_OK) return COBRA_ECUDA;
+  coords_kernel<<<dim3((unsigned)((n_tok + kCoordTok - 1) / kCoordTok), (unsigned)n_heads), kAppendThreads,
+                  proj_smem_bytes(), s>>>(a);
   if (cudaGetLastError() != cudaSuccess) return COBRA_ECUDA;
-  measure_kernel<<<dim3((unsigned)n_r, (unsigned)n_heads), 256, 0, s>>>(a);
+  measure_kernel<<<dim3((unsigned)n_r, (unsigned)n_heads), kMeasureThreads, 0, s>>>(a);
   return launch_status();
 }
 

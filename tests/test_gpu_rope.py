@@ -82,3 +82,27 @@ def test_positions_outside_the_table_are_reported():
     with pytest.raises(AssertionError):
         run_decode(params, srcs, 1, 2, 4, [200], rope=dict(theta=LLAMA3_THETA, q_pos=[5000], max_pos=256))
     assert cobra.cobra_check() == cobra.COBRA_OK  # the status word was read and cleared
+
+
+@pytest.mark.parametrize("G,bk,bv", [(4, 4, 4), (4, 6, 5), (4, 8, 8), (8, 5, 6), (8, 8, 8)])
+def test_wide_rows_in_every_staging_form(G, bk, bv):
+    """Full-rank rows: two stages per warpgroup, one, and a single warpgroup (r = 128 at 8 bits on
+    both sides), over several rows and a partial last one."""
+    rbs = [(128, bk), (126, bk), (128, bv), (110, bv)]
+    params, srcs = mixed_heads(2, rbs, cfg=51)
+    o, ref, _ = run_decode(params, srcs, 1, 2, G, [1500, 130], rope=dict(theta=LLAMA3_THETA))
+    assert rel_err(o, ref) < TOL
+
+
+def test_takes_that_run_over_several_groups():
+    """More plan chunks than CTAs take one at a time: a take crosses sequences and heads."""
+    rbs = [(34, 2), (16, 1), (20, 3), (48, 2)]
+    params, srcs = mixed_heads(2, rbs, cfg=52)
+    g = np.random.default_rng(3)
+    lens = [int(x) for x in g.integers(0, 300, 400)]
+    o, ref, info = run_decode(params, srcs, 1, 2, 4, lens, cap=[300] * len(lens),
+                              rope=dict(theta=LLAMA3_THETA, max_pos=300))
+    assert info.n_items > 4 * 152
+    live = [i for i, t in enumerate(lens) if t]
+    assert rel_err(o[:, live], ref[:, live]) < TOL
+    assert np.all(np.delete(o, live, axis=1) == 0)
