@@ -359,7 +359,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const int r = he.r, b = he.b;
   const int nrows = (a.n_tok + kRowTokens - 1) / kRowTokens;
   const int ntiles = a.n_seqs * nrows;
-  if (r == 0 || chunk >= ntiles) return;
+  grid_dep_launch();
+  if (r == 0 || chunk >= ntiles) {
+    grid_dep_wait();
+    return;
+  }
   const int my_tiles = (ntiles - chunk + a.chunks - 1) / a.chunks;
   const int nsplit = b >= 6 ? 3 : 2;
   const float* pool = param_pool(a.block);
@@ -390,6 +394,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
+    grid_dep_wait();  // X may be the result of a kernel ahead
     if (lane == 0) {
       int issued = 0;
       for (int i = 0; i < my_tiles; ++i) {
@@ -419,6 +424,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: Y^T[128 channels][128 tokens] per tile ----------------
+    grid_dep_wait();
     if (lane == 0) {
       const uint32_t idesc = umma_idesc_bf16(128, 128);
       const uint32_t xbase = smem_addr(xsm);
@@ -464,12 +470,15 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // channels >= r are zero.
     {
       const float4* wrow = reinterpret_cast<const float4*>(pool + he.w_off + (size_t)(ch < r ? ch : 0) * kD);
-#pragma unroll 1
+      float4 wv[32];  // the whole row in flight at once
+#pragma unroll
+      for (int u = 0; u < 32; ++u) wv[u] = ch < r ? wrow[u] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
       for (int q = 0; q < 4; ++q) {
         float rem[32];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          const float4 f = ch < r ? wrow[8 * q + u] : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 f = wv[8 * q + u];
           rem[4 * u] = f.x;
           rem[4 * u + 1] = f.y;
           rem[4 * u + 2] = f.z;
@@ -494,6 +503,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(WREADY));
     }
+    grid_dep_wait();  // kernels ahead may still read the cache rows written below
     TcEpi e;
     const float scale = 1.0f / (float)(1 << b);  // a power of two: the scaled values are exact
     e.inv_s = he.inv_delta * scale;

@@ -65,6 +65,27 @@ cobra_status ensure_smem(Kernel kernel, size_t bytes, Granted& granted) {
 }  // namespace
 
 namespace {
+// Launch with programmatic stream serialisation: the kernel may become resident while the one
+// ahead of it in the stream finishes; it waits for that kernel (grid_dep_wait) before touching
+// anything the kernel ahead may produce or read.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                       Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+}  // namespace
+
+namespace {
 
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -178,33 +199,20 @@ extern "C" cobra_status cobra_compress(const void* params, const cobra_compress_
       chunks = c;
     }
   }
+  // Too few tiles for 16 per CTA on every SM (a chunk of one layer's prefill): one wave of as many
+  // CTAs as there are SMs or tiles instead, however few tiles each gets.  K and V of 1 layer x 8 kv
+  // heads x 2001 tokens: 14 us for both calls on 128 CTAs each, 50 on 8.
+  if (heads * std::max(1LL, tiles / 16) < sms) chunks = std::max(1LL, std::min(tiles, sms / heads));
   a.chunks = (int)chunks;
   const long long grid = heads * chunks;
   if (grid > 0x7fffffffLL) return COBRA_EINVAL;
-  compress_tc_kernel<<<(unsigned)grid, kTcThreads, kTcSmemBytes, (cudaStream_t)stream>>>(map, a);
+  // its setup (barriers, TMEM, the basis) overlaps the end of the kernel ahead
+  if (launch_pdl(compress_tc_kernel, (unsigned)grid, kTcThreads, kTcSmemBytes, (cudaStream_t)stream, map, a) !=
+      cudaSuccess)
+    return COBRA_ECUDA;
   return launch_status();
 }
 
-namespace {
-// Launch with programmatic stream serialisation: the kernel may become resident while the one
-// ahead of it in the stream finishes; it waits for that kernel (grid_dep_wait) before touching
-// anything the kernel ahead may produce or read.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
-                       Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-}  // namespace
 
 namespace {
 // How the sequences of each (layer, kv head) are spread over projecting CTAs (append, query

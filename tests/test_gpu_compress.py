@@ -198,3 +198,22 @@ def test_compress_head_major_layers_padded_tokens():
             for q in range(seqs):
                 check_head(host, offs[l * H + h], 0, params[l * H + h], xs[l, h, q, :, :128], T, seq=q,
                            rows_per_seq=nrows)
+
+
+@pytest.mark.parametrize("H,S,T", [(1, 1, 129), (2, 3, 3461), (5, 1, 2048), (3, 40, 130), (8, 1, 2001)])
+def test_few_tiles_spread_over_ctas(H, S, T):
+    """Calls with fewer tiles than fill every SM at 16 per CTA spread them over more CTAs: the same
+    bytes as with the sequences and heads compressed one at a time (one tile per CTA, or few)."""
+    srcs = [synth.HeadSource(71, 0, h, 0, (0.3, 2.5)) for h in range(H)]
+    params = [oracle_head(s, r, b) for s, (r, b) in zip(srcs, [(128, 4), (34, 7), (64, 2), (18, 1), (100, 3)] * 2)]
+    g = np.random.default_rng(S)
+    xs = g.standard_normal((S, T, H, 128)).astype(np.float32)
+    rows = -(-T // 128)
+    for side in (0, 1):
+        host, offs, r, b, _ = run_compress(params, srcs, T, side, seqs=S, x_override=xs)
+        for q in (0, S // 2, S - 1):
+            one, o1, *_ = run_compress(params, srcs, T, side, seqs=1, x_override=xs[q:q + 1])
+            for h in range(H):
+                rb = 16 * int(r[h]) * int(b[h])
+                a = host[int(offs[h]) + q * rows * rb:][:rows * rb]
+                assert np.array_equal(a, one[int(o1[h]):][:rows * rb])
