@@ -812,8 +812,10 @@ extern "C" cobra_status cobra_calibrate_heads(int n_heads, int n_tok, const floa
   if (!aligned(x, 4) || (q && !aligned(q, 4)) || !aligned(mu, 8) || !aligned(lam, 8) || !aligned(U, 8) ||
       !aligned(w, 8))
     return COBRA_EALIGN;
-  static Granted granted;
-  if (ensure_smem(calib_kernel, calib_smem_bytes(), granted) != COBRA_OK) return COBRA_ECUDA;
+  static Granted mom_granted, eig_granted;
+  if (ensure_smem(moments_kernel, moments_smem_bytes(), mom_granted) != COBRA_OK ||
+      ensure_smem(eigen_kernel, eigen_smem_bytes(), eig_granted) != COBRA_OK)
+    return COBRA_ECUDA;
   CalibArgs a{};
   a.x = x;
   a.q = n_q > 0 ? q : nullptr;
@@ -823,7 +825,11 @@ extern "C" cobra_status cobra_calibrate_heads(int n_heads, int n_tok, const floa
   a.w = w;
   a.n_tok = n_tok;
   a.n_q = n_q;
-  calib_kernel<<<(unsigned)n_heads, kCalThreads, calib_smem_bytes(), (cudaStream_t)stream>>>(a);
+  const long long grid = (long long)n_heads * kMomParts * (a.q ? 2 : 1);
+  if (grid > 0x7fffffffLL) return COBRA_EINVAL;
+  moments_kernel<<<(unsigned)grid, kMomThreads, moments_smem_bytes(), (cudaStream_t)stream>>>(a);
+  if (cudaGetLastError() != cudaSuccess) return COBRA_ECUDA;
+  eigen_kernel<<<(unsigned)n_heads, kEigThreads, eigen_smem_bytes(), (cudaStream_t)stream>>>(a);
   return launch_status();
 }
 

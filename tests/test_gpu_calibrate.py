@@ -68,3 +68,38 @@ def test_device_calibration_feeds_the_same_allocation():
         a = cobra.cobra_allocate(np.stack([c["w"] for c in dev[part]]), 1.0)
         b = cobra.cobra_allocate(np.stack([c["w"] for c in host[part]]), 1.0)
         assert np.array_equal(a["r"], b["r"]) and np.array_equal(a["b"], b["b"])
+
+
+@pytest.mark.parametrize("n_tok,n_q,n", [(1, 0, 1), (2, 3, 2), (31, 33, 1), (100, 1, 3), (128, 0, 2), (130, 64, 1), (700, 37, 5)])
+def test_device_calibration_of_any_rank(n_tok, n_q, n):
+    """Rank-deficient heads (fewer vectors than dimensions, equal vectors): the directions of a
+    multiple eigenvalue are not unique, so the check is of what defines a decomposition - orthonormal
+    directions that give the covariance back to rounding (512 eps of its norm; the pivoted factor of a
+    singular matrix is of the matrix plus a shift of 2^-40 of its largest entry)."""
+    g = np.random.default_rng(n_tok)
+    A = g.standard_normal((n, 128, 128)) * (np.arange(1, 129) ** -1.3)[None, None, :]
+    x = (g.standard_normal((n, n_tok, 128)) @ A.transpose(0, 2, 1) + 0.5).astype(np.float32)
+    x[-1, n_tok // 2:] = x[-1, 0]  # the last head holds the same vector over and over
+    q = g.standard_normal((n, n_q, 128)).astype(np.float32) if n_q else None
+    xd = torch.tensor(x, device=DEV)
+    qd = torch.tensor(q, device=DEV) if n_q else None
+    f64 = lambda *s: torch.full(s, float("nan"), dtype=torch.float64, device=DEV)
+    mu, lam, U, w = f64(n, 128), f64(n, 128), f64(n, 128 * 128), f64(n, 128)
+    cobra.cobra_calibrate_heads(xd, qd, mu, lam, U, w)
+    torch.cuda.synchronize()
+    mu, lam, U, w = mu.cpu().numpy(), lam.cpu().numpy(), U.cpu().numpy().reshape(n, 128, 128), w.cpu().numpy()
+    for h in range(n):
+        xh = x[h].astype(np.float64)
+        c = xh - xh.mean(axis=0)
+        cov = c.T @ c / n_tok
+        norm = np.linalg.norm(cov)
+        np.testing.assert_allclose(mu[h], xh.mean(axis=0), rtol=0, atol=1e-12 * max(1.0, np.abs(xh).max()))
+        assert np.abs(U[h] @ U[h].T - np.eye(128)).max() < 512 * 2.2e-16
+        assert np.abs(U[h].T @ (lam[h][:, None] * U[h]) - cov).max() <= max(512 * 2.2e-16, 2.0 ** -40) * norm + 1e-300
+        assert np.all(np.diff(w[h]) <= 0)
+        assert all(u[np.argmax(np.abs(u))] > 0 for u in U[h])
+        if n_q:
+            var = ((q[h].astype(np.float64) @ U[h].T) ** 2).mean(axis=0)
+            np.testing.assert_allclose(w[h], var * lam[h], rtol=1e-9, atol=1e-12 * max(np.abs(w[h]).max(), 1e-300))
+        else:
+            assert np.array_equal(w[h], lam[h])
