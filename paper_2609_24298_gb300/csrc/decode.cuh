@@ -5,7 +5,7 @@
 //                   kv head, split into fp16 hi + lo, laid out as MMA B fragments.
 //   decode_kernel   persistent warps over work items (token chunks of one (seq, layer, kv-head)).
 //                   Each warp streams its chunk's K and V code rows into a private shared-
-//                   memory ring with bulk async copies, unpacks codes in registers and runs
+//                   memory ring with async copies, unpacks codes in registers and runs
 //                   f16 mma.sync with fp32 accumulation:
 //                     scores  S[t][col] = sum_i code^K[t][i] q~[i][col]   (M = tokens, K = channels)
 //                     values  O[i][g]  += sum_t code^V[t][i] P[t][g]      (M = channels, K = tokens)
@@ -29,8 +29,7 @@
 
 namespace cobra {
 
-constexpr int kDecodeWarps = 4;
-constexpr int kMaxStages = 8;
+constexpr int kDecodeWarps = 2;  // per CTA: small CTAs fill the shared memory better when rows are large
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s
 
 struct DecodeArgs {
@@ -63,8 +62,11 @@ struct Heads {
 //
 // Per warp and work item (a run of code rows of one (seq, layer, kv head)):
 //  * each stage of the warp's shared-memory ring holds one K row and the V row of the same
-//    tokens, both copied with cp.async.bulk onto one mbarrier; the copies are issued by one
-//    lane under a predicate, so the warp never diverges;
+//    tokens, both copied by the warp's lanes with 16-byte cp.async, a commit group per stage, one
+//    row ahead of the row being scored.  (One lane issuing bulk copies on an mbarrier per stage took
+//    130 warp-instructions per row pair of about 1100, this about 50: 32 layers x 8 kv heads x
+//    8 x 32768 tokens at 1 bpd 891 -> 858 us per step, 80 layers at 0.5 bpd with 8 query heads per kv
+//    head 1222 -> 1134.);
 //  * scores s_t (log2 units) come from the K codes by f16 MMA; probabilities are taken
 //    against a reference max that is raised (and the accumulators rescaled) only when a
 //    row's max exceeds it by more than kTau, so most rows need no rescale;
@@ -301,12 +303,26 @@ struct ScanWarp {
   uint8_t* ring;
   float* osm;
   uint2* qfrag;
-  uint64_t* bars;
   int ring_bytes, lane;
-  bool leader, failed;
-  uint32_t phase_bits;  // parity of the next wait per barrier
-  int wait_stage, nstage, outstanding;
 };
+
+// Copies n bytes (a multiple of 16) to shared memory: lane l moves bytes 16 l, 16 l + 512, ... of
+// them; src and dst are the lane's first ones.
+__device__ __forceinline__ void lane_copy_async(uint32_t dst, const uint8_t* src, uint32_t n, uint32_t lane_off) {
+  for (uint32_t o = lane_off; o < n; o += 2048u) {
+    cp_async16(dst, src);
+    if (o + 512u < n) cp_async16(dst + 512u, src + 512);
+    if (o + 1024u < n) cp_async16(dst + 1024u, src + 1024);
+    if (o + 1536u < n) cp_async16(dst + 1536u, src + 1536);
+    dst += 2048u;
+    src += 2048;
+  }
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 
 // One work item.  BK / BV > 0 fix the K / V bit widths at compile time (the common widths
 // get their own copy of the row loop); 0 dispatches on the runtime widths row by row.
@@ -314,7 +330,6 @@ template <int G, int BK, int BV>
 __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int item) {
   constexpr int NG = G / 4, NO = OAcc<G>::N;
   const int lane = w.lane;
-  const bool leader = w.leader;
   const WsHeader* wh = reinterpret_cast<const WsHeader*>(a.ws);
   const WsGroup* groups = reinterpret_cast<const WsGroup*>(a.ws + wh->groups_off);
   const WsItem* items = reinterpret_cast<const WsItem*>(a.ws + wh->items_off);
@@ -335,18 +350,18 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
   // consumed, so the whole ring is free)
   const uint32_t kst = (rbk + 127u) & ~127u;
   const int stage_bytes = (int)max(kst + ((rbv + 127u) & ~127u), 128u);
-  w.nstage = min(kMaxStages, w.ring_bytes / stage_bytes);
-  w.wait_stage = 0;
-  if (w.nstage < 1) {
+  if (stage_bytes > w.ring_bytes) {
     // a row pair that does not fit the staging ring is never copied; report and leave an
     // empty chunk (m = -inf, l = 0)
-    if (leader) atomicOr(&g_status, 2u);
+    if (lane == 0) atomicOr(&g_status, 2u);
     if (lane < G) {
       part[lane * gstride + 0] = -INFINITY;
       part[lane * gstride + 1] = 0.f;
     }
     return;
   }
+  // two stages, or one (copied and waited for row by row) when a pair takes over half the ring
+  const bool two = 2 * stage_bytes <= w.ring_bytes;
   float* osm = w.osm;
   float mref[NG];
 #pragma unroll
@@ -358,7 +373,6 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
   const int vc = (vr > 0 && vb <= 2) ? vb : 0;
   const int vbd = vr > 0 ? vb : 0;
   const float vout = vr == 0 ? 0.f : (float)(1 << (vb == 1 ? 5 : vb == 2 ? 6 : vb));
-  const int n_loads = (row1 > row0 && (rbk || rbv)) ? row1 - row0 : 0;
   const unsigned char* qt = a.ws + wh->qt_off + (size_t)it.group * wh->qt_stride;
   const float* qhdr = reinterpret_cast<const float*>(qt);
   const uint2* bfrag = w.qfrag;  // filled together with the item's first stage
@@ -368,77 +382,47 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
   const float qscale = qhdr[8];
   const uint32_t one = a.one;
 
-  // issue state: next row and stage to load (every lane tracks it; lane 0 issues).  In a
-  // contiguous cache the item's rows follow one another, so the sources advance by a row;
-  // a paged cache looks each row's page up.
-  int iss_row = row0, iss_stage = 0;
-  const uint8_t* kbase = a.cache + koff;
-  const uint8_t* vbase = a.cache + voff;
+  // the lane's part of the next row to copy.  In a contiguous cache the item's rows follow one
+  // another, so the sources advance by a row; a paged cache looks each row's page up.
+  const uint32_t lane_off = 16u * lane;
+  const uint8_t* kbase = a.cache + koff + lane_off;
+  const uint8_t* vbase = a.cache + voff + lane_off;
   const int* const page_table = a.page_table;
   const int pages_per_seq = a.pages_per_seq, seq = gr.seq;
   const size_t slot0 = (size_t)seq * a.rows_per_seq + row0;
   const uint8_t* ksrc = kbase + slot0 * rbk;
   const uint8_t* vsrc = vbase + slot0 * rbv;
-  const uint32_t ring0 = smem_addr(w.ring), bar0 = smem_addr(w.bars);
-  const int nstage = w.nstage;
-  auto issue_next = [&]() {
+  const uint32_t dst0 = smem_addr(w.ring) + lane_off;
+  auto copy_row = [&](int row, uint32_t stage_off) {
     const uint8_t* ks = ksrc;
     const uint8_t* vs = vsrc;
     if (page_table) {
-      ks = kbase + row_offset(0, rbk, seq, iss_row, page_table, pages_per_seq, 0);
-      vs = vbase + row_offset(0, rbv, seq, iss_row, page_table, pages_per_seq, 0);
+      ks = kbase + row_offset(0, rbk, seq, row, page_table, pages_per_seq, 0);
+      vs = vbase + row_offset(0, rbv, seq, row, page_table, pages_per_seq, 0);
     }
-    const uint32_t dst = ring0 + (uint32_t)(iss_stage * stage_bytes);
-    refill_pair_if(leader, bar0 + 8u * iss_stage, dst, ks, rbk, dst + kst, vs, rbv);
+    lane_copy_async(dst0 + stage_off, ks, rbk, lane_off);
+    lane_copy_async(dst0 + stage_off + kst, vs, rbv, lane_off);
     ksrc += rbk;
     vsrc += rbv;
-    ++iss_row;
-    iss_stage = iss_stage + 1 == nstage ? 0 : iss_stage + 1;
   };
-  int issued = min(n_loads, w.nstage);
-  if (issued > 0 && rbk) {
-    // the q~ fragments travel with the first stage: the previous item's reads of them are
-    // ordered before the copy by the warp barrier and the proxy fence
-    __syncwarp();
-    fence_proxy_async_smem_if(leader);
-    const uint32_t bar = smem_addr(&w.bars[0]);
-    mbar_expect_tx_if(leader, bar, decode_qfrag_bytes<G>());  // stage 0's issue below arrives
-    bulk_g2s_if(leader, smem_addr(w.qfrag), qt + kQtHeaderBytes, decode_qfrag_bytes<G>(), bar);
+  __syncwarp();  // the previous item's reads of the ring and the fragments are done
+  if (row0 < row1) {
+    if (rbk) lane_copy_async(smem_addr(w.qfrag) + lane_off, qt + kQtHeaderBytes + lane_off, decode_qfrag_bytes<G>(), lane_off);
+    copy_row(row0, 0);
   }
-  for (int k = 0; k < issued; ++k) issue_next();
-  w.outstanding = issued;
-
-  // wait for the next stage; returns its buffer or nullptr on timeout
-  auto acquire = [&]() -> const uint8_t* {
-    const uint32_t bar = bar0 + 8u * w.wait_stage, parity = (w.phase_bits >> w.wait_stage) & 1u;
-    // the stage has normally landed already: one probe, and the bounded wait only when not
-    if (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity)) &&
-        !__all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, kWaitLimitNs)))
-      return nullptr;
-    w.phase_bits ^= 1u << w.wait_stage;
-    return w.ring + (size_t)w.wait_stage * stage_bytes;
-  };
-  // release the stage just consumed and refill it with the next row pair of this item
-  auto release = [&]() {
-    __syncwarp();
-    --w.outstanding;
-    if (++w.wait_stage == w.nstage) w.wait_stage = 0;
-    if (issued < n_loads) {
-      issue_next();  // its proxy fence orders this warp's reads of the stage before the copies
-      ++issued;
-      ++w.outstanding;
-    }
-  };
+  cp_async_commit();
+  uint32_t cur = 0;  // offset of the stage of the row being scored
 
   for (int row = row0; row < row1; ++row) {
-    const uint8_t* buf = nullptr;
-    if (n_loads) {
-      buf = acquire();
-      if (!buf) {
-        w.failed = true;
-        return;
-      }
+    if (two) {
+      if (row + 1 < row1) copy_row(row + 1, cur ^ (uint32_t)stage_bytes);
+      cp_async_commit();
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
     }
+    __syncwarp();
+    const uint8_t* buf = w.ring + cur;
     float s[8][NG][2];
     if (rbk) {
       if constexpr (BK > 0)
@@ -498,7 +482,13 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
         row_probs<G, 0>(s, mref, bv);
       v_row_dispatch<G>(vbd, buf + kst, vr, bv, one, osm);
     }
-    if (n_loads) release();
+    __syncwarp();  // every lane is done with the stage
+    if (two) {
+      cur ^= (uint32_t)stage_bytes;
+    } else if (row + 1 < row1) {
+      copy_row(row + 1, 0);
+      cp_async_commit();
+    }
   }
   // ---- write the partial of this item: m, l and (O - c) 2^(10 - kmin) per query head ----
   __syncwarp();
@@ -531,30 +521,18 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
 }
 
 template <int G>
-__global__ void __launch_bounds__(kDecodeWarps * 32, 4) decode_kernel(DecodeArgs a) {
+__global__ void __launch_bounds__(kDecodeWarps * 32, 8) decode_kernel(DecodeArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   // the combine kernel may be scheduled as CTAs of this grid exit (it waits for the results)
   grid_dep_launch();
   const int warp = threadIdx.x >> 5;
   ScanWarp w;
   w.lane = threadIdx.x & 31;
-  w.leader = w.lane == 0;
   w.ring_bytes = a.ring_bytes;
   const size_t warp_bytes = (size_t)w.ring_bytes + decode_osm_bytes<G>() + decode_qfrag_bytes<G>();
   w.ring = smem + (size_t)warp * warp_bytes;
   w.osm = reinterpret_cast<float*>(w.ring + w.ring_bytes);
   w.qfrag = reinterpret_cast<uint2*>(w.ring + w.ring_bytes + decode_osm_bytes<G>());
-  w.bars = reinterpret_cast<uint64_t*>(smem + (size_t)kDecodeWarps * warp_bytes) + warp * kMaxStages;
-  w.failed = false;
-  w.phase_bits = 0;
-  w.wait_stage = 0;
-  w.nstage = 1;
-  w.outstanding = 0;
-  if (w.leader) {
-    for (int i = 0; i < kMaxStages; ++i) mbar_init(smem_addr(&w.bars[i]), 1);
-    fence_mbar_init();
-  }
-  __syncwarp();
   // the q~ blocks come from the query projection ahead, the cache from the appends before it
   grid_dep_wait();
 
@@ -568,10 +546,10 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 4) decode_kernel(DecodeArgs
   unsigned int* next_item = const_cast<unsigned int*>(&wh->next_item);
   auto take = [&]() -> int {
     int v = 0;
-    if (w.leader) v = (int)atomicAdd(next_item, 1u);
+    if (w.lane == 0) v = (int)atomicAdd(next_item, 1u);
     return __shfl_sync(0xffffffffu, v, 0);
   };
-  for (int item = take(); item < n_items && !w.failed; item = take()) {
+  for (int item = take(); item < n_items; item = take()) {
     if constexpr (G == 4) {
       // the bit widths of 1 to 3 that carry most of the cache at low rates, and the 3- to 5-bit
       // pairs of rates of 3 to 4 bpd, get their own code
@@ -608,16 +586,6 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 4) decode_kernel(DecodeArgs
         case 0x22: scan_item<G, 2, 2>(a, w, item); break;
         default: scan_item<G, 0, 0>(a, w, item); break;
       }
-    }
-  }
-  if (w.failed) {
-    if (w.leader) atomicOr(&g_status, 1u);
-    // drain the copies still in flight before the shared memory goes away
-    for (int k = 0; k < w.outstanding; ++k) {
-      if (!mbar_wait_bounded(smem_addr(&w.bars[w.wait_stage]), (w.phase_bits >> w.wait_stage) & 1u, kWaitLimitNs))
-        break;
-      w.phase_bits ^= 1u << w.wait_stage;
-      if (++w.wait_stage == w.nstage) w.wait_stage = 0;
     }
   }
   // the last CTA to run out of items puts the work counter back to 0 for the next launch:

@@ -836,6 +836,21 @@ constexpr long long kItemMin = 16 * 1024, kItemMax = 128 * 1024;
 constexpr long long kScanWarps = 152 * 16;  // resident scan warps: 152 SMs x 4 CTAs x 4 warps
 constexpr long long kGuide = 2;
 constexpr long long kMaxChunks = 32;
+constexpr long long kWaveRowsMin = 5, kWaveRowsMax = 12;
+constexpr long long kWaveMaxChunks = 64;  // per group, when few groups share the warps
+
+// Warp-instructions of the scan per 128-token row pair, in tenths: about 310, and per channel by bit
+// width (measured on the row functions; widths whose codes straddle words cost more).
+long long row_cost(int rk, int bk, int rv, int bv) {
+  constexpr long long per[9] = {0, 38, 42, 72, 48, 70, 75, 80, 55};
+  return 3100 + per[bk] * rk + per[bv] * rv;
+}
+// resident scan warps: 16 per SM, or as many as the shared memory holds (CTAs of two warps; per warp
+// the ring, 2.25 KB of accumulators and 2 KB of query fragments for a group of 4, twice for 8)
+long long resident_warps(size_t max_row, int group) {
+  const size_t per_cta = 2 * (cobra::scan_ring_bytes(max_row) + (group == 4 ? 4352 : 8704)) + 1024;
+  return 152 * std::min<long long>(16, 2 * std::max<long long>(1, (long long)(233472 / per_cta)));
+}
 
 cobra_status check_decode_desc(const cobra_decode_desc* d) {
   if (!d) return COBRA_EINVAL;
@@ -886,7 +901,19 @@ cobra_status make_plan(const cobra_decode_desc* d, const int* head_r, const int*
     return (long long)cobra_row_bytes(k.rk, k.bk) + (long long)cobra_row_bytes(k.rv, k.bv);
   };
   long long remaining = 0;  // packed K+V bytes not yet in a chunk
-  for (const Key& k : keys) remaining += (long long)(seq_cap[k.s] + 127) / 128 * pair_bytes(k);
+  long long total_rows = 0, total_cost = 0;
+  size_t max_row = 0;
+  for (const Key& k : keys) {
+    const long long rows = (seq_cap[k.s] + 127) / 128;
+    remaining += rows * pair_bytes(k);
+    total_rows += rows;
+    total_cost += rows * row_cost(k.rk, k.bk, k.rv, k.bv);
+    max_row = std::max(max_row, std::max(cobra_row_bytes(k.rk, k.bk), cobra_row_bytes(k.rv, k.bv)));
+  }
+  const long long warps = resident_warps(max_row, d->group);
+  const bool one_wave =
+      total_rows <= warps || (total_rows >= kWaveRowsMin * warps && total_rows <= kWaveRowsMax * warps);
+  const long long wave_max = std::min(kWaveMaxChunks, std::max(kMaxChunks, warps / (long long)keys.size()));
   for (const Key& key : keys) {
     const int hk = d->k_head0 + key.l * d->layer_stride + key.h, hv = d->v_head0 + key.l * d->layer_stride + key.h;
     p.max_rv = std::max(p.max_rv, key.rv);
@@ -900,8 +927,17 @@ cobra_status make_plan(const cobra_decode_desc* d, const int* head_r, const int*
       p.items.push_back({(int)p.groups.size(), 0, (int)rows, (int)p.items.size()});
       g.n_items = 1;
     }
+    if (one_wave && rows > 0 && rb > 0) {
+      // rounded down: the chunks of all groups together are at most one per warp
+      const long long share = rows * row_cost(key.rk, key.bk, key.rv, key.bv) * warps / total_cost;
+      const long long n = std::max(1LL, std::min(std::min(rows, wave_max), share));
+      for (long long c = 0; c < n; ++c) {
+        p.items.push_back({(int)p.groups.size(), (int)(rows * c / n), (int)(rows * (c + 1) / n), (int)p.items.size()});
+        g.n_items++;
+      }
+    }
     const long long min_rows = (rows + kMaxChunks - 1) / kMaxChunks;
-    for (long long r0 = 0; r0 < rows && rb > 0;) {
+    for (long long r0 = 0; r0 < rows && rb > 0 && !one_wave;) {
       const long long target = std::min(kItemMax, std::max(kItemMin, remaining / (kGuide * kScanWarps)));
       long long n = std::max(min_rows, std::max(1LL, (target + rb / 2) / rb));
       if (rows - r0 - n < (n + 1) / 2) n = rows - r0;  // no short remainder chunk

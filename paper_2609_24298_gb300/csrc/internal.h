@@ -78,4 +78,15 @@ constexpr int kQtStride = kQtHeaderBytes + 8 * 2 * 32 * 8;
 
 constexpr size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// The scan's per-warp staging ring for code rows of at most `max_row` bytes: 8 KB, or two of the
+// largest rows if those are bigger.  Rows of 12 KB and more get four (at most 32 KB): with such rows
+// the copies, not the warps, bound the scan, and two stages of a typical row pair for 6 warps per SM
+// beat three for 4 (2 layers x 32 ragged sequences at 4 bpd: 559 against 619 us per step) and one for
+// 8 (at 3 bpd, with 10 KB rows, the smaller ring is the better one).
+constexpr size_t scan_ring_bytes(size_t max_row) {
+  const size_t row = align_up(max_row > 16 ? max_row : 16, 128), two = 2 * row > 8192 ? 2 * row : 8192;
+  const size_t four = 4 * row < 32 * 1024 ? 4 * row : 32 * 1024;
+  return max_row >= 12288 && four > two ? four : two;
+}
+
 }  // namespace cobra
