@@ -521,7 +521,7 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
 }
 
 template <int G>
-__global__ void __launch_bounds__(kDecodeWarps * 32, 8) decode_kernel(DecodeArgs a) {
+__global__ void __launch_bounds__(kDecodeWarps * 32, G == 4 ? 8 : 6) decode_kernel(DecodeArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   // the combine kernel may be scheduled as CTAs of this grid exit (it waits for the results)
   grid_dep_launch();
@@ -541,12 +541,18 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 8) decode_kernel(DecodeArgs
   const WsItem* items = reinterpret_cast<const WsItem*>(a.ws + wh->items_off);
   const HeadEntry* heads = head_table(a.block);
   const int n_items = wh->n_items;
-  // work items are taken in plan order from a shared counter, so that warps that finish early
-  // take more (the items' costs differ with the heads' bit widths)
+  // work items are taken in plan order from a shared counter, so that warps that finish early take
+  // more (the items' costs differ with the heads' bit widths).  When every item has a warp of its
+  // own, warp 0 of every CTA has one before warp 1 of any (few items spread over the SMs) and the
+  // counter is not asked; with more items that would put different code variants on an SM.
   unsigned int* next_item = const_cast<unsigned int*>(&wh->next_item);
+  int own = n_items <= (int)(kDecodeWarps * gridDim.x) ? (int)(blockIdx.x + warp * gridDim.x) : -1;
   auto take = [&]() -> int {
-    int v = 0;
-    if (w.lane == 0) v = (int)atomicAdd(next_item, 1u);
+    int v = own;
+    if (own >= 0)
+      own = n_items;
+    else if (w.lane == 0)
+      v = (int)atomicAdd(next_item, 1u);
     return __shfl_sync(0xffffffffu, v, 0);
   };
   for (int item = take(); item < n_items; item = take()) {

@@ -310,8 +310,8 @@ cobra_status launch_decode(const DecodeArgs& a, int n_heads, int n_seqs, int n_i
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_kernel<G>, kDecodeWarps * 32, smem) != cudaSuccess)
       return COBRA_ECUDA;
     per_sm = std::max(per_sm, 1);
-    const int want = (n_items + kDecodeWarps - 1) / kDecodeWarps;
-    const int grid = std::max(1, std::min(want, per_sm * sm_count()));
+    // one item per CTA while SMs are free (a CTA's other warps then find none)
+    const int grid = std::max(1, std::min(n_items, per_sm * sm_count()));
     // the work counter is 0 here: the plan writes it so, and every scan's last CTA resets it
     if (launch_pdl(decode_kernel<G>, (unsigned)grid, kDecodeWarps * 32, smem, s, a) != cudaSuccess) return COBRA_ECUDA;
   }

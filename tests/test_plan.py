@@ -141,3 +141,40 @@ def test_plan_host_reports_size_without_buffer():
     assert info.n_groups == 8 and img.size > 128
     with pytest.raises(RuntimeError):
         cobra.cobra_decode_plan_host(d, r, b, [4096])  # beyond rows_per_seq
+
+
+@pytest.mark.parametrize("S,T,rb,rows_per_chunk", [
+    (1, 2048, (128, 2), (1, 1)),       # fewer rows than warps: a warp per row
+    (8, 32768, (64, 2), (6, 8)),       # a layer of long sequences: one chunk per warp
+    (8, 32768, (64, 3), (6, 8)),
+    (3, 131072, (64, 2), (16, 17)),    # few groups: at most 64 chunks each
+    (24, 2944, (64, 3), None),         # between the two: chunks of at least 16 KB, taken as warps free up
+])
+def test_plan_of_one_layer_fills_one_wave(S, T, rb, rows_per_chunk):
+    H = 8
+    r, b = np.full(2 * H, rb[0], np.int32), np.full(2 * H, rb[1], np.int32)
+    d, img, info = make(1, H, S, [T] * S, r, b)
+    h, g, it, hg = parse(img)
+    rows = T // 128
+    for gi, (s, l, kv, first, n, hk, hv, _) in enumerate(g):
+        mine = it[it[:, 0] == gi]
+        assert len(mine) == n and np.array_equal(np.sort(mine[:, 3]), np.arange(first, first + n))
+        spans = mine[np.argsort(mine[:, 1]), 1:3]
+        assert spans[0, 0] == 0 and spans[-1, 1] == rows and np.all(spans[1:, 0] == spans[:-1, 1])
+    size = it[:, 2] - it[:, 1]
+    if rows_per_chunk:
+        assert size.min() >= rows_per_chunk[0] and size.max() <= rows_per_chunk[1]
+        assert len(it) <= 152 * 16 and g[:, 4].max() <= 64
+    else:
+        assert size.min() >= 1 and len(it) > 152 * 8
+
+
+def test_plan_of_one_layer_weighs_the_widths():
+    """Heads of equal bytes but different widths: 1-bit rows cost the scan more and get more chunks."""
+    H, S = 8, 8
+    r = np.array([128, 64] * 8, np.int32)
+    b = np.array([1, 2] * 8, np.int32)
+    d, img, info = make(1, H, S, [32768] * S, r, b)
+    h, g, it, hg = parse(img)
+    n1, n2 = g[b[g[:, 5]] == 1, 4], g[b[g[:, 5]] == 2, 4]
+    assert n1.min() > 1.2 * n2.max() and g[:, 4].sum() <= 152 * 16
