@@ -214,7 +214,24 @@ __device__ __forceinline__ void v_row_accumulate(const uint8_t* stage, int rv, c
   };
 #pragma unroll 1
   for (int mu = 0; mu < nfull; ++mu) tile(false, mu);
-  tile(true, nfull);
+  if (P & 7) {
+    tile(true, nfull);
+  } else {
+    // only the constant rows: row 0 of the tile (1.0) and row 1 (the window factors)
+    float d[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    const bool nrm = B <= 2 && (lane >> 2) == 1;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const uint32_t a0 = nrm ? unshift_h2<B>(2 * t) : one, a2 = nrm ? unshift_h2<B>(2 * t + 1) : one;
+      mma_f16(d[t & 1], a0, one, a2, one, bv[t][0], bv[t][1]);
+    }
+    if constexpr (NO == 2) {
+      o[0] += d[0][0] + d[1][0];
+    } else {
+      o[0] += d[0][0] + d[1][0];
+      o[1] += d[0][1] + d[1][1];
+    }
+  }
 }
 
 template <int G>
@@ -445,24 +462,29 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
           if (tbase + 16 * t + 8 >= T) s[t][u][1] = -INFINITY;
         }
     }
-    // row max per head; the reference max moves (and the accumulators are rescaled) only
-    // when it is exceeded by more than kTau
-    bool move = false;
-    float alpha[NG];
+    // the reference max moves (and the accumulators are rescaled) only when a score exceeds it by
+    // more than kTau: one vote per row, the row max only then
+    float mx[NG];
+    bool exceed = false;
 #pragma unroll
     for (int u = 0; u < NG; ++u) {
-      float mx = -INFINITY;
+      mx[u] = -INFINITY;
 #pragma unroll
-      for (int t = 0; t < 8; ++t) mx = fmaxf(mx, fmaxf(s[t][u][0], s[t][u][1]));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-      const bool mv = mx > mref[u] + kTau;
-      alpha[u] = mv ? ex2_approx(mref[u] - mx) : 1.f;
-      mref[u] = mv ? mx : mref[u];
-      move |= mv;
+      for (int t = 0; t < 8; ++t) mx[u] = fmaxf(mx[u], fmaxf(s[t][u][0], s[t][u][1]));
+      exceed |= mx[u] > mref[u] + kTau;
     }
-    if (__any_sync(0xffffffffu, move)) {
+    if (__any_sync(0xffffffffu, exceed)) {
+      float alpha[NG];
+#pragma unroll
+      for (int u = 0; u < NG; ++u) {
+        float m = mx[u];
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 4));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+        const bool mv = m > mref[u] + kTau;
+        alpha[u] = mv ? ex2_approx(mref[u] - m) : 1.f;
+        mref[u] = mv ? m : mref[u];
+      }
       for (int mu = 0; mu < ntile; ++mu) {
         float* o = osm + (mu * 32 + lane) * NO;
 #pragma unroll
