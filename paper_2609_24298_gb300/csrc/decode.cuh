@@ -29,7 +29,7 @@
 
 namespace cobra {
 
-constexpr int kDecodeWarps = 2;  // per CTA: small CTAs fill the shared memory better when rows are large
+constexpr int kDecodeWarps = 4;  // per CTA at most (see scan_shape)
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s
 
 struct DecodeArgs {
@@ -43,6 +43,7 @@ struct DecodeArgs {
   long long q_sl, q_ss, o_sl, o_ss;
   int rows_per_seq, pages_per_seq;
   int ring_bytes;  // per-warp staging ring (>= 2 of the largest code rows, multiple of 128)
+  int n_sms;
   uint32_t one;    // kOneH2, passed at run time so that it stays in a register
 };
 
@@ -276,6 +277,10 @@ template <int G>
 __host__ __device__ constexpr uint32_t decode_qfrag_bytes() {
   return 8u * Heads<G>::NTK * 32u * 8u;
 }
+
+static_assert(decode_osm_bytes<4>() + decode_qfrag_bytes<4>() == scan_state_bytes(4) &&
+                  decode_osm_bytes<8>() + decode_qfrag_bytes<8>() == scan_state_bytes(8),
+              "the plan counts on the scan's shared memory");
 
 // VC is the V bit width's window class: 0 = one window for every register (b >= 3, or no V
 // codes), 1 or 2 = the b = 1 / b = 2 windows.  V codes read 1 + code * 2^(k-10) with a
@@ -543,7 +548,7 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
 }
 
 template <int G>
-__global__ void __launch_bounds__(kDecodeWarps * 32, G == 4 ? 8 : 6) decode_kernel(DecodeArgs a) {
+__global__ void __launch_bounds__(kDecodeWarps * 32, G == 4 ? 4 : 3) decode_kernel(DecodeArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   // the combine kernel may be scheduled as CTAs of this grid exit (it waits for the results)
   grid_dep_launch();
@@ -566,9 +571,17 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, G == 4 ? 8 : 6) decode_kern
   // work items are taken in plan order from a shared counter, so that warps that finish early take
   // more (the items' costs differ with the heads' bit widths).  When every item has a warp of its
   // own, warp 0 of every CTA has one before warp 1 of any (few items spread over the SMs) and the
-  // counter is not asked; with more items that would put different code variants on an SM.
+  // counter is not asked; with more items that would put different code variants on an SM.  CTAs b,
+  // b + n_sms, ... are resident on one SM as a rule and take neighbouring items, which share their
+  // code and their group's query fragments.
   unsigned int* next_item = const_cast<unsigned int*>(&wh->next_item);
-  int own = n_items <= (int)(kDecodeWarps * gridDim.x) ? (int)(blockIdx.x + warp * gridDim.x) : -1;
+  int own = -1;
+  if (n_items <= (int)((blockDim.x >> 5) * gridDim.x)) {
+    const int n_sms = gridDim.x % a.n_sms == 0 ? a.n_sms : (int)gridDim.x;  // not full: item b for CTA b
+    const int per = (n_items + n_sms - 1) / n_sms, sm = (int)blockIdx.x % n_sms;
+    const int k = (int)blockIdx.x / n_sms + warp * ((int)gridDim.x / n_sms);
+    own = k < per ? sm * per + k : n_items;
+  }
   auto take = [&]() -> int {
     int v = own;
     if (own >= 0)

@@ -845,13 +845,6 @@ long long row_cost(int rk, int bk, int rv, int bv) {
   constexpr long long per[9] = {0, 38, 42, 72, 48, 70, 75, 80, 55};
   return 3100 + per[bk] * rk + per[bv] * rv;
 }
-// resident scan warps: 16 per SM, or as many as the shared memory holds (CTAs of two warps; per warp
-// the ring, 2.25 KB of accumulators and 2 KB of query fragments for a group of 4, twice for 8)
-long long resident_warps(size_t max_row, int group) {
-  const size_t per_cta = 2 * (cobra::scan_ring_bytes(max_row) + (group == 4 ? 4352 : 8704)) + 1024;
-  return 152 * std::min<long long>(16, 2 * std::max<long long>(1, (long long)(233472 / per_cta)));
-}
-
 cobra_status check_decode_desc(const cobra_decode_desc* d) {
   if (!d) return COBRA_EINVAL;
   if (d->n_layers < 1 || d->n_kv_heads < 1 || d->n_seqs < 1 || (d->group != 4 && d->group != 8) ||
@@ -910,7 +903,7 @@ cobra_status make_plan(const cobra_decode_desc* d, const int* head_r, const int*
     total_cost += rows * row_cost(k.rk, k.bk, k.rv, k.bv);
     max_row = std::max(max_row, std::max(cobra_row_bytes(k.rk, k.bk), cobra_row_bytes(k.rv, k.bv)));
   }
-  const long long warps = resident_warps(max_row, d->group);
+  const long long warps = 152LL * cobra::scan_shape(cobra::scan_ring_bytes(max_row), d->group).sm_warps;
   const bool one_wave =
       total_rows <= warps || (total_rows >= kWaveRowsMin * warps && total_rows <= kWaveRowsMax * warps);
   const long long wave_max = std::min(kWaveMaxChunks, std::max(kMaxChunks, warps / (long long)keys.size()));

@@ -89,4 +89,26 @@ constexpr size_t scan_ring_bytes(size_t max_row) {
   return max_row >= 12288 && four > two ? four : two;
 }
 
+// The scan's shared memory per warp besides the ring: V accumulators and query fragments.
+constexpr size_t scan_state_bytes(int group) { return group == 4 ? 4352 : 8704; }
+
+// Warps per scan CTA and resident warps per SM (at most 16, the registers' limit): 4, 2 or 1 warps,
+// whichever fits the most into 228 KB of shared memory (1 KB of it per CTA is the system's); the
+// larger CTA of equals, whose launches are fewer.  A layer of 8 kv heads x 8 x 32768 tokens at 1 bpd
+// (8 KB rings) takes 57 us per step with 4, 60 with 2 and 65 with 1; 2 layers x 32 ragged sequences at
+// 4 bpd (32 KB rings) 639, 547 and 541.
+struct ScanShape {
+  int cta_warps, sm_warps;
+};
+constexpr ScanShape scan_shape(size_t ring, int group) {
+  ScanShape best{1, 0};
+  for (int nw = 4; nw >= 1; nw /= 2) {
+    const size_t cta = nw * (ring + scan_state_bytes(group)) + 1024;
+    const size_t n = nw * (233472 / cta);
+    const int warps = n < 16 ? (int)n : 16;
+    if (warps > best.sm_warps) best = ScanShape{nw, warps};
+  }
+  return best;
+}
+
 }  // namespace cobra

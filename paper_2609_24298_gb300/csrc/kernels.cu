@@ -302,18 +302,18 @@ cobra_status launch_decode(const DecodeArgs& a, int n_heads, int n_seqs, int n_i
     }
   }
   if (stages & kScan) {
-    const size_t smem =
-        (size_t)kDecodeWarps * ((size_t)a.ring_bytes + decode_osm_bytes<G>() + decode_qfrag_bytes<G>());
+    const int nw = scan_shape((size_t)a.ring_bytes, G).cta_warps;
+    const size_t smem = (size_t)nw * ((size_t)a.ring_bytes + scan_state_bytes(G));
     static Granted granted;
     if (ensure_smem(decode_kernel<G>, smem, granted) != COBRA_OK) return COBRA_ECUDA;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_kernel<G>, kDecodeWarps * 32, smem) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_kernel<G>, nw * 32, smem) != cudaSuccess)
       return COBRA_ECUDA;
     per_sm = std::max(per_sm, 1);
     // one item per CTA while SMs are free (a CTA's other warps then find none)
     const int grid = std::max(1, std::min(n_items, per_sm * sm_count()));
     // the work counter is 0 here: the plan writes it so, and every scan's last CTA resets it
-    if (launch_pdl(decode_kernel<G>, (unsigned)grid, kDecodeWarps * 32, smem, s, a) != cudaSuccess) return COBRA_ECUDA;
+    if (launch_pdl(decode_kernel<G>, (unsigned)grid, (unsigned)(nw * 32), smem, s, a) != cudaSuccess) return COBRA_ECUDA;
   }
   if (stages & kCombine) {
     // one CTA per (layer, kv head, sequence); its prologue (the plan, the L2 prefetch of W_V)
@@ -357,6 +357,7 @@ cobra_status decode_args(const void* params, const cobra_decode_desc* d, const c
   a.rows_per_seq = d->rows_per_seq;
   a.pages_per_seq = d->pages_per_seq;
   a.one = kOneH2;
+  a.n_sms = sm_count();
   a.ring_bytes = (int)scan_ring_bytes((size_t)info->max_row_bytes);
   const long long n_heads = (long long)d->n_layers * d->n_kv_heads;
   if (n_heads * d->n_seqs != info->n_groups) return COBRA_EINVAL;  // plan made for another descriptor
@@ -717,6 +718,7 @@ extern "C" cobra_status cobra_decode_attn_static(const void* params, const cobra
   a.rows_per_seq = d->rows_per_seq;
   a.pages_per_seq = d->pages_per_seq;
   a.one = kOneH2;
+  a.n_sms = sm_count();
   a.ring_bytes = 2 * 16 * kD * 8;  // two rows of the largest head (r = 128, b = 8)
   const int n_heads = d->n_layers * d->n_kv_heads;
   if (d->group == 4) return launch_decode<4>(a, n_heads, d->n_seqs, (int)n_groups, kQproj | kScan | kCombine, s, true);
