@@ -62,12 +62,14 @@ struct Heads {
 // a5 + a6: chunked rank-space scan
 //
 // Per warp and work item (a run of code rows of one (seq, layer, kv head)):
-//  * each stage of the warp's shared-memory ring holds one K row and the V row of the same
-//    tokens, both copied by the warp's lanes with 16-byte cp.async, a commit group per stage, one
-//    row ahead of the row being scored.  (One lane issuing bulk copies on an mbarrier per stage took
-//    130 warp-instructions per row pair of about 1100, this about 50: 32 layers x 8 kv heads x
-//    8 x 32768 tokens at 1 bpd 891 -> 858 us per step, 80 layers at 0.5 bpd with 8 query heads per kv
-//    head 1222 -> 1134.);
+//  * the warp's shared-memory ring holds one K row and the V row of the same tokens, copied by its
+//    lanes with 16-byte cp.async, a commit group per row: the next K row is copied while the warp
+//    works on the V row and the next V row while it works on the next K row, so that half a row pair
+//    of work covers a copy and the ring is no larger than a pair.  (One lane issuing bulk copies on
+//    an mbarrier per stage took 130 warp-instructions per row pair of about 1100.  Two stages of
+//    whole pairs left 6 warps per SM at 4 bpd and single-buffered rows at 3: 539 against 453 us per
+//    step for 2 layers x 32 ragged sequences at 4 bpd, 817 against 795 for 32 layers x 8 x 32768
+//    tokens at 1 bpd.);
 //  * scores s_t (log2 units) come from the K codes by f16 MMA; probabilities are taken
 //    against a reference max that is raised (and the accumulators rescaled) only when a
 //    row's max exceeds it by more than kTau, so most rows need no rescale;
@@ -368,11 +370,10 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
   const int row0 = it.row_begin, row1 = min(it.row_end, rows_valid);
   float* part = parts + (size_t)it.slot * pstride;
   const uint32_t rbk = kr > 0 ? 16u * kr * kb : 0u, rbv = vr > 0 ? 16u * vr * vb : 0u;
-  // one stage = this item's K row + V row (every load of the previous item has been
-  // consumed, so the whole ring is free)
-  const uint32_t kst = (rbk + 127u) & ~127u;
-  const int stage_bytes = (int)max(kst + ((rbv + 127u) & ~127u), 128u);
-  if (stage_bytes > w.ring_bytes) {
+  // the ring holds one K row and one V row (every load of the previous item has been consumed)
+  const uint32_t kst = (rbk + 127u) & ~127u;  // the V row's place in the ring
+  const int pair_bytes = (int)(kst + ((rbv + 127u) & ~127u));
+  if (pair_bytes > w.ring_bytes) {
     // a row pair that does not fit the staging ring is never copied; report and leave an
     // empty chunk (m = -inf, l = 0)
     if (lane == 0) atomicOr(&g_status, 2u);
@@ -382,8 +383,6 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
     }
     return;
   }
-  // two stages, or one (copied and waited for row by row) when a pair takes over half the ring
-  const bool two = 2 * stage_bytes <= w.ring_bytes;
   float* osm = w.osm;
   float mref[NG];
 #pragma unroll
@@ -415,36 +414,30 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
   const uint8_t* ksrc = kbase + slot0 * rbk;
   const uint8_t* vsrc = vbase + slot0 * rbv;
   const uint32_t dst0 = smem_addr(w.ring) + lane_off;
-  auto copy_row = [&](int row, uint32_t stage_off) {
-    const uint8_t* ks = ksrc;
-    const uint8_t* vs = vsrc;
-    if (page_table) {
-      ks = kbase + row_offset(0, rbk, seq, row, page_table, pages_per_seq, 0);
-      vs = vbase + row_offset(0, rbv, seq, row, page_table, pages_per_seq, 0);
-    }
-    lane_copy_async(dst0 + stage_off, ks, rbk, lane_off);
-    lane_copy_async(dst0 + stage_off + kst, vs, rbv, lane_off);
+  auto copy_k = [&](int row) {
+    const uint8_t* ks = page_table ? kbase + row_offset(0, rbk, seq, row, page_table, pages_per_seq, 0) : ksrc;
+    lane_copy_async(dst0, ks, rbk, lane_off);
     ksrc += rbk;
+  };
+  auto copy_v = [&](int row) {
+    const uint8_t* vs = page_table ? vbase + row_offset(0, rbv, seq, row, page_table, pages_per_seq, 0) : vsrc;
+    lane_copy_async(dst0 + kst, vs, rbv, lane_off);
     vsrc += rbv;
   };
   __syncwarp();  // the previous item's reads of the ring and the fragments are done
   if (row0 < row1) {
     if (rbk) lane_copy_async(smem_addr(w.qfrag) + lane_off, qt + kQtHeaderBytes + lane_off, decode_qfrag_bytes<G>(), lane_off);
-    copy_row(row0, 0);
+    copy_k(row0);
+    cp_async_commit();
+    copy_v(row0);
+    cp_async_commit();
   }
-  cp_async_commit();
-  uint32_t cur = 0;  // offset of the stage of the row being scored
 
   for (int row = row0; row < row1; ++row) {
-    if (two) {
-      if (row + 1 < row1) copy_row(row + 1, cur ^ (uint32_t)stage_bytes);
-      cp_async_commit();
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
+    // groups in flight: this row's K, this row's V
+    cp_async_wait<1>();
     __syncwarp();
-    const uint8_t* buf = w.ring + cur;
+    const uint8_t* buf = w.ring;
     float s[8][NG][2];
     if (rbk) {
       if constexpr (BK > 0)
@@ -457,6 +450,9 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
 #pragma unroll
         for (int u = 0; u < NG; ++u) s[t][u][0] = s[t][u][1] = 0.f;
     }
+    __syncwarp();  // every lane is done with the K row
+    if (row + 1 < row1) copy_k(row + 1);
+    cp_async_commit();
     if ((row + 1) * kRowTokens > T) {  // only the last row of a sequence has masked tokens
       const int tbase = row * kRowTokens + (lane >> 2);
 #pragma unroll
@@ -497,6 +493,9 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
       }
     }
     uint32_t bv[8][2];
+    // groups in flight: this row's V, the next row's K
+    cp_async_wait<1>();
+    __syncwarp();
     if constexpr (BV > 0) {
       row_probs<G, (BV <= 2 ? BV : 0)>(s, mref, bv);
       v_row_accumulate<G, BV>(buf + kst, vr, bv, one, osm);
@@ -509,13 +508,9 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
         row_probs<G, 0>(s, mref, bv);
       v_row_dispatch<G>(vbd, buf + kst, vr, bv, one, osm);
     }
-    __syncwarp();  // every lane is done with the stage
-    if (two) {
-      cur ^= (uint32_t)stage_bytes;
-    } else if (row + 1 < row1) {
-      copy_row(row + 1, 0);
-      cp_async_commit();
-    }
+    __syncwarp();  // every lane is done with the V row
+    if (row + 1 < row1) copy_v(row + 1);
+    cp_async_commit();
   }
   // ---- write the partial of this item: m, l and (O - c) 2^(10 - kmin) per query head ----
   __syncwarp();

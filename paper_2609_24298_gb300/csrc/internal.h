@@ -78,15 +78,10 @@ constexpr int kQtStride = kQtHeaderBytes + 8 * 2 * 32 * 8;
 
 constexpr size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// The scan's per-warp staging ring for code rows of at most `max_row` bytes: 8 KB, or two of the
-// largest rows if those are bigger.  Rows of 12 KB and more get four (at most 32 KB): with such rows
-// the copies, not the warps, bound the scan, and two stages of a typical row pair for 6 warps per SM
-// beat three for 4 (2 layers x 32 ragged sequences at 4 bpd: 559 against 619 us per step) and one for
-// 8 (at 3 bpd, with 10 KB rows, the smaller ring is the better one).
+// The scan's per-warp staging ring for code rows of at most `max_row` bytes: a K and a V row.
 constexpr size_t scan_ring_bytes(size_t max_row) {
-  const size_t row = align_up(max_row > 16 ? max_row : 16, 128), two = 2 * row > 8192 ? 2 * row : 8192;
-  const size_t four = 4 * row < 32 * 1024 ? 4 * row : 32 * 1024;
-  return max_row >= 12288 && four > two ? four : two;
+  const size_t two = 2 * align_up(max_row, 128);
+  return two > 8192 ? two : 8192;
 }
 
 // The scan's shared memory per warp besides the ring: V accumulators and query fragments.
@@ -96,7 +91,7 @@ constexpr size_t scan_state_bytes(int group) { return group == 4 ? 4352 : 8704; 
 // whichever fits the most into 228 KB of shared memory (1 KB of it per CTA is the system's); the
 // larger CTA of equals, whose launches are fewer.  A layer of 8 kv heads x 8 x 32768 tokens at 1 bpd
 // (8 KB rings) takes 57 us per step with 4, 60 with 2 and 65 with 1; 2 layers x 32 ragged sequences at
-// 4 bpd (32 KB rings) 639, 547 and 541.
+// 4 bpd (24 to 32 KB rings) 639, 547 and 541.
 struct ScanShape {
   int cta_warps, sm_warps;
 };
