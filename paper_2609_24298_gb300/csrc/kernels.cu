@@ -464,6 +464,15 @@ int smem_optin() {
   return n;
 }
 
+template <int G, int MAXWG>
+cobra_status launch_rope_wg(const DecodeArgs& a, RopeArgs ra, int nwg, size_t smem, int grid, cudaStream_t s) {
+  static Granted granted;
+  if (ensure_smem(rope_scan_kernel<G, MAXWG>, smem, granted) != COBRA_OK) return COBRA_ECUDA;
+  const cudaError_t e =
+      launch_pdl(rope_scan_kernel<G, MAXWG>, (unsigned)grid, (unsigned)(160 * nwg), smem, s, a, ra);
+  return e == cudaSuccess ? COBRA_OK : COBRA_ECUDA;
+}
+
 template <int G>
 cobra_status launch_rope(const DecodeArgs& a, const RopeArgs& ra0, int n_heads, int n_seqs, int n_items,
                          int max_row_bytes, int max_stage_bytes, cudaStream_t s) {
@@ -475,26 +484,29 @@ cobra_status launch_rope(const DecodeArgs& a, const RopeArgs& ra0, int n_heads, 
                                           : align_up(rowb + 1792, 128) + align_up(rowb, 128);
   const size_t stage = std::max<size_t>(align_up(need, 128), 128);
   ra.stage_bytes = (int)stage;
-  // two warpgroups with two stages each where they fit (up to about 4 bits per dimension on both
-  // sides), else with one stage, else one warpgroup
-  const size_t fixed = rope_fixed_bytes<G>();
-  const long long room = (long long)smem_optin() - (long long)fixed;
-  const long long fit = room > 0 ? room / (long long)stage : 0;
-  if (fit < 1) return COBRA_EINVAL;  // code rows too large for the staging
-  const int nwg = fit >= 2 ? 2 : 1;
-  ra.n_stage = fit >= 2 * nwg ? 2 : 1;
-  const size_t smem = fixed + (size_t)(nwg * ra.n_stage) * stage;
-  static Granted granted;
-  if (ensure_smem(rope_scan_kernel<G>, smem, granted) != COBRA_OK) return COBRA_ECUDA;
-  // chunks taken at a time: W_K is staged again for each take, so a call that does not fill the GPU
-  // four times over is dealt out in one take per CTA, a larger one in four or more (the chunks
-  // shrink towards the end of the plan).  The work counter is 0 here (the plan writes it so, every
-  // scan resets it).
+  // three warpgroups with two stages each where they fit (up to about 2 bits per dimension on both
+  // sides), two with two (4 bits), with one, else one warpgroup
+  auto fit = [&](int nwg) {  // stages that fit beside nwg warpgroups' buffers
+    const long long room = (long long)smem_optin() - (long long)rope_fixed_bytes<G>(nwg);
+    return room > 0 ? room / (long long)stage : 0;
+  };
   const int sms = sm_count();
-  ra.batch = n_items <= 4 * sms ? (n_items + sms - 1) / sms : (n_items + 4 * sms - 1) / (4 * sms);
+  const int nwg = G == 4 && n_items > 4 * sms && fit(3) >= 6 ? 3 : fit(2) >= 2 ? 2 : 1;
+  if (fit(nwg) < nwg) return COBRA_EINVAL;  // code rows too large for the staging
+  ra.n_stage = fit(nwg) >= 2 * nwg ? 2 : 1;
+  const size_t smem = rope_fixed_bytes<G>(nwg) + (size_t)(nwg * ra.n_stage) * stage;
+  // chunks taken at a time: W_K is staged again for each take, so a call that does not fill the GPU
+  // four times over is dealt out in one take per CTA, a larger one in six or more (the chunks
+  // shrink towards the end of the plan; a take costs about 6 us of staging and draining).  The work counter is 0 here (the plan writes it so, every
+  // scan resets it).
+  ra.batch = n_items <= 4 * sms ? (n_items + sms - 1) / sms : (n_items + 6 * sms - 1) / (6 * sms);
   const int grid = std::max(1, std::min((n_items + ra.batch - 1) / ra.batch, sms));
-  if (launch_pdl(rope_scan_kernel<G>, (unsigned)grid, (unsigned)(160 * nwg), smem, s, a, ra) != cudaSuccess)
-    return COBRA_ECUDA;
+  cobra_status st;
+  if constexpr (G == 4)
+    st = nwg == 3 ? launch_rope_wg<4, 3>(a, ra, nwg, smem, grid, s) : launch_rope_wg<4, 2>(a, ra, nwg, smem, grid, s);
+  else
+    st = launch_rope_wg<8, 2>(a, ra, nwg, smem, grid, s);
+  if (st != COBRA_OK) return st;
   return launch_decode<G>(a, n_heads, n_seqs, n_items, kCombine, s);
 }
 

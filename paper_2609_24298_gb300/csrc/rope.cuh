@@ -12,7 +12,7 @@
 //   rope_table_kernel  cos and sin of x omega_j in fp64, for x = i < 16 (fine rows) and
 //                      x = 16 m (coarse rows); any position x = 16 m + i composes from one of
 //                      each by the angle-addition formulas.
-//   rope_scan_kernel   CTAs of one or two warpgroups, each with a warp that issues its MMAs and
+//   rope_scan_kernel   CTAs of one to three warpgroups, each with a warp that issues its MMAs and
 //                      copies, take runs of the decode plan's chunks; a warpgroup takes every other
 //                      128-token row of a run.  Per row, with thread t owning token t (TMEM lane t):
 //                        unpack   the token's codes, as f16, into TMEM (the MMAs' A operand)
@@ -49,7 +49,11 @@ namespace cobra {
 
 constexpr int kRopeFine = 16;         // positions per coarse step (fine rows 0..15)
 constexpr int kRopeRowFloats = 128;   // floats per table row: [jj 4][n 16][cos, sin]
-constexpr int kRopeMaxWg = 2;         // warpgroups (128 threads) per CTA
+// Warpgroups (128 threads and an issuing warp) per CTA at most.  Three cap a thread at 128 registers,
+// which 4 query heads fit but for a few spills: calls of many rows gain from the third warpgroup (4
+// layers x 8 heads x 8 x 32768 tokens at 1 bpd: 943 against 998 us), short ones lose more to the cap
+// (34.8 against 32.5 us for 1 x 8191) and use the build with two; 8 query heads always do.
+constexpr int kRopeMaxWg = 3;
 // A raised reference lies this far below the maximum, so that fewer of the small probabilities fall
 // into fp16's subnormals (fed values stay below 2^kTau).
 constexpr float kRopeLift = 4.f;
@@ -89,19 +93,19 @@ struct RopeWgSmem {
 };
 template <int G>
 struct RopeSmem {
-  RopeWgSmem<G> wg[kRopeMaxWg];
   float4 qbase[32 * G];         // R(p) q, scaled
-  float merge[G][4 + kD];       // m, l, -, -, O of the second warpgroup
+  float merge[kRopeMaxWg - 1][G][4 + kD];  // m, l, -, -, O of the warpgroups after the first
   uint32_t tmem;
   int batch, fail;
+  alignas(16) RopeWgSmem<G> wg[1];  // one per warpgroup
 };
 template <int G>
-__host__ __device__ constexpr size_t rope_vars_bytes() {
-  return (sizeof(RopeSmem<G>) + 127) / 128 * 128;
+__host__ __device__ constexpr size_t rope_vars_bytes(int nwg) {
+  return (sizeof(RopeSmem<G>) + (nwg - 1) * sizeof(RopeWgSmem<G>) + 127) / 128 * 128;
 }
 template <int G>
-__host__ __device__ constexpr size_t rope_fixed_bytes() {
-  return 1024 + kRopeWBytes + kRopeTrigBytes + rope_vars_bytes<G>();
+__host__ __device__ constexpr size_t rope_fixed_bytes(int nwg) {
+  return 1024 + kRopeWBytes + kRopeTrigBytes + rope_vars_bytes<G>(nwg);
 }
 
 // (cos, sin) of x omega_j for x = 16 m + i from the coarse (m) and fine (i) entries
@@ -336,8 +340,8 @@ __device__ __forceinline__ void rope_v_dispatch(int b, const uint8_t* vrow, int 
 // over stretches of consecutive rows of one group (W_K is staged when the K head changes); the
 // stretch's sums go to its first chunk's slot and its other chunks are left empty.
 // ---------------------------------------------------------------------------------------
-template <int G>
-__global__ void __launch_bounds__(kRopeMaxWg * 160, 1) rope_scan_kernel(DecodeArgs a, RopeArgs ra) {
+template <int G, int MAXWG>
+__global__ void __launch_bounds__(MAXWG * 160, 1) rope_scan_kernel(DecodeArgs a, RopeArgs ra) {
   constexpr int NO = OAcc<G>::N;
   extern __shared__ uint8_t smem_raw[];
   // the combine kernel may be scheduled as CTAs of this grid exit (it waits for the results)
@@ -346,7 +350,6 @@ __global__ void __launch_bounds__(kRopeMaxWg * 160, 1) rope_scan_kernel(DecodeAr
   uint8_t* wsm = smem_raw + (((raw + 1023u) & ~1023u) - raw);  // W' hi atoms 0..2, lo atoms 3, 4
   float4* trig = reinterpret_cast<float4*>(wsm + kRopeWBytes);
   RopeSmem<G>& sh = *reinterpret_cast<RopeSmem<G>*>(wsm + kRopeWBytes + kRopeTrigBytes);
-  uint8_t* stages = wsm + kRopeWBytes + kRopeTrigBytes + rope_vars_bytes<G>();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // the compute warps of all warpgroups, then one warp per warpgroup that issues MMAs and copies
   const int nwg = blockDim.x / 160;
@@ -354,7 +357,7 @@ __global__ void __launch_bounds__(kRopeMaxWg * 160, 1) rope_scan_kernel(DecodeAr
   const int wg = mma_warp ? warp - 4 * nwg : tid >> 7, wq = warp & 3, t = tid & 127;
   RopeWgSmem<G>& ws = sh.wg[wg];
   const int ns = ra.n_stage;
-  uint8_t* stage0 = stages + (size_t)wg * ns * ra.stage_bytes;
+  uint8_t* stage0 = wsm + kRopeWBytes + kRopeTrigBytes + rope_vars_bytes<G>(nwg) + (size_t)wg * ns * ra.stage_bytes;
   const uint32_t bar0 = smem_addr(ws.bars);
   auto bar_k = [&](int i) { return bar0 + 8u * i; };
   auto bar_v = [&](int i) { return bar0 + 16u + 8u * i; };
@@ -393,7 +396,6 @@ __global__ void __launch_bounds__(kRopeMaxWg * 160, 1) rope_scan_kernel(DecodeAr
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sh.tmem;
-  const uint32_t x_col = tmem + 128u * wg, a_col = tmem + 256u + 128u * wg;  // this warpgroup's X and A
   const uint32_t lanes = (uint32_t)(32 * wq) << 16;                          // this warp's TMEM lanes
   const float4* trig_t = trig + t;
   const uint32_t one = a.one;
@@ -452,21 +454,24 @@ __global__ void __launch_bounds__(kRopeMaxWg * 160, 1) rope_scan_kernel(DecodeAr
       const int row1 = last_slot == gr.first_item + gr.n_items - 1 ? min(rows_valid, cap_rows) : min(rows_valid, row_end);
       const uint32_t rbk = rk > 0 ? 16u * rk * kb : 0u, rbv = vr > 0 ? 16u * vr * vb : 0u;
       const uint32_t kst = rk > 0 ? 256u * kb * nk : 0u;  // whole channel tiles (the last may read past the row)
+      // TMEM's 512 columns hold X (128) and A (8 nk + 8) of three warpgroups up to nk = 4, of two beyond
+      const int nact = nk <= 4 ? nwg : min(nwg, 2);
+      const uint32_t x_col = tmem + 128u * wg, a_col = tmem + 128u * nact + (nact == 3 ? 40u : 72u) * wg;
       const bool fits = kst + ((rbv + 127u) & ~127u) <= (uint32_t)ra.stage_bytes;
       if (!fits && tid == 0) atomicOr(&g_status, 2u);
       if (T > kRopeFine * ra.n_coarse && tid == 0) atomicOr(&g_status, 2u);  // positions past the table
-      const int n_rows = fits && row1 > row0 + wg ? (row1 - row0 - wg + nwg - 1) / nwg : 0;  // of this warpgroup
+      const int n_rows = fits && wg < nact && row1 > row0 + wg ? (row1 - row0 - wg + nact - 1) / nact : 0;  // of this warpgroup
       const uint8_t* kbase = a.cache + hk.cache_off;
       const uint8_t* vbase = a.cache + hv.cache_off;
       // copies of the n-th row's K or V into its stage (one thread)
       auto load_k = [&](int n) {
-        const int st = n % ns, row = row0 + wg + n * nwg;
+        const int st = n % ns, row = row0 + wg + n * nact;
         mbar_arrive_expect_tx(bar_k(st), rbk);
         bulk_g2s(smem_addr(stage0 + (size_t)st * ra.stage_bytes),
                  kbase + row_offset(0, rbk, gr.seq, row, a.page_table, a.pages_per_seq, a.rows_per_seq), rbk, bar_k(st));
       };
       auto load_v = [&](int n) {
-        const int st = n % ns, row = row0 + wg + n * nwg;
+        const int st = n % ns, row = row0 + wg + n * nact;
         mbar_arrive_expect_tx(bar_v(st), rbv);
         bulk_g2s(smem_addr(stage0 + (size_t)st * ra.stage_bytes + kst),
                  vbase + row_offset(0, rbv, gr.seq, row, a.page_table, a.pages_per_seq, a.rows_per_seq), rbv, bar_v(st));
@@ -500,7 +505,7 @@ __global__ void __launch_bounds__(kRopeMaxWg * 160, 1) rope_scan_kernel(DecodeAr
         }
         // the constant A columns: 1 in the first three elements of tile nk
         const uint32_t cst[8] = {0x3C003C00u, 0x00003C00u, 0u, 0u, 0u, 0u, 0u, 0u};
-        tc_st32x8(a_col + lanes + 8 * nk, cst);
+        if (wg < nact) tc_st32x8(a_col + lanes + 8 * nk, cst);
         tc_wait_st();
         tc_fence_before();
         if (wg == 0) {  // mu' / Delta in three limbs
@@ -565,7 +570,7 @@ __global__ void __launch_bounds__(kRopeMaxWg * 160, 1) rope_scan_kernel(DecodeAr
       constexpr int QN = G / 4;
       float2 ang[QN][2];
       auto load_angles = [&](int n) {
-        const float* crs = coarse + (size_t)min(8 * (row0 + wg + n * nwg), ra.n_coarse - 1) * kRopeRowFloats;
+        const float* crs = coarse + (size_t)min(8 * (row0 + wg + n * nact), ra.n_coarse - 1) * kRopeRowFloats;
 #pragma unroll
         for (int u = 0; u < QN; ++u)
 #pragma unroll
@@ -701,7 +706,7 @@ __global__ void __launch_bounds__(kRopeMaxWg * 160, 1) rope_scan_kernel(DecodeAr
           wg_sync(wg);  // publishes the first row's query
         }
         for (int n = 0; n < n_rows; ++n) {
-          const int row = row0 + wg + n * nwg;
+          const int row = row0 + wg + n * nact;
           const uint32_t par = (uint32_t)(total + n) & 1u;
           const float4* q = ws.q[n & 1];
           f32x2 acc[2 * G];
@@ -778,39 +783,42 @@ __global__ void __launch_bounds__(kRopeMaxWg * 160, 1) rope_scan_kernel(DecodeAr
           }
         }
       };
-      if (wg == 1 && !mma_warp) {
-        entries([&](int g, int ch, float v) { sh.merge[g][4 + ch] = v; });
+      if (wg > 0 && wg < nact && !mma_warp) {
+        entries([&](int g, int ch, float v) { sh.merge[wg - 1][g][4 + ch] = v; });
         if (t == 0) {
 #pragma unroll
           for (int g = 0; g < G; ++g) {
-            sh.merge[g][0] = mref[g];
-            sh.merge[g][1] = lsum[g];
+            sh.merge[wg - 1][g][0] = mref[g];
+            sh.merge[wg - 1][g][1] = lsum[g];
           }
         }
       }
       __syncthreads();
       if (wg == 0 && !mma_warp) {
         float* part = parts + (size_t)it0.slot * pstride;
+        // e: the entry of a warpgroup's block (1: l, 4 + channel: O); v0: this warpgroup's value
+        auto merged = [&](int g, float m0, int e, float v0, float& M) {
+          M = m0;
+          for (int x = 0; x < nact - 1; ++x) M = fmaxf(M, sh.merge[x][g][0]);
+          float r = m0 != -INFINITY ? exp2f(m0 - M) * v0 : 0.f;
+          for (int x = 0; x < nact - 1; ++x)
+            if (sh.merge[x][g][0] != -INFINITY) r += exp2f(sh.merge[x][g][0] - M) * sh.merge[x][g][e];
+          return r;
+        };
         if (t == 0) {
 #pragma unroll
           for (int g = 0; g < G; ++g) {
-            const float m1 = nwg > 1 ? sh.merge[g][0] : -INFINITY, M = fmaxf(mref[g], m1);
-            float l = 0.f;
-            if (mref[g] != -INFINITY) l += exp2f(mref[g] - M) * lsum[g];
-            if (m1 != -INFINITY) l += exp2f(m1 - M) * sh.merge[g][1];
+            float M;
+            const float l = merged(g, mref[g], 1, lsum[g], M);
             part[g * gstride] = M;
             part[g * gstride + 1] = l;
           }
         }
         entries([&](int g, int ch, float v) {
-          float m0 = mref[0];
+          float m0 = mref[0], M;
 #pragma unroll
           for (int k = 1; k < G; ++k) m0 = g == k ? mref[k] : m0;
-          const float m1 = nwg > 1 ? sh.merge[g][0] : -INFINITY, M = fmaxf(m0, m1);
-          float x = 0.f;
-          if (m0 != -INFINITY) x += exp2f(m0 - M) * v;
-          if (m1 != -INFINITY) x += exp2f(m1 - M) * sh.merge[g][4 + ch];
-          part[g * gstride + 4 + ch] = x;
+          part[g * gstride + 4 + ch] = merged(g, m0, 4 + ch, v, M);
         });
         for (int i = i0 + 1 + t / G; i < i1; i += 128 / G) {  // the stretch's other chunks
           float* pg = parts + (size_t)items[i].slot * pstride + (t % G) * gstride;
