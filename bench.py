@@ -402,7 +402,8 @@ def run_compress_leg(args, dev, stream, peak):
 
 
 MEASURE_PROFILE = os.path.join(ROOT, "profiles", "measure_tables_llama3_8b.txt")
-MEASURE_SOURCES = ["paper_2609_24298_gb300/csrc/measure.cuh", "paper_2609_24298_gb300/csrc/common.cuh"]
+MEASURE_SOURCES = ["paper_2609_24298_gb300/csrc/measure.cuh", "paper_2609_24298_gb300/csrc/compress.cuh",
+                   "paper_2609_24298_gb300/csrc/common.cuh"]
 ISSUE_PEAK = 152 * 4 * 2.07e9  # warp-instructions per second: 152 SMs x 4 schedulers at 2070 MHz
 
 
@@ -483,9 +484,9 @@ def run_calibration_leg(args, dev, stream, srcs, cpu_baseline: bool):
         "unit": "ms for all heads", "higher_is_better": False,
         "workload": f"{len(srcs)} heads (32 layers x 8 kv heads x K/V) x 512 calibration vectors; K heads with "
                     f"{G * 512} calibration queries each",
-        "calls": K, "launches": 2 * K,
+        "calls": K, "launches": 4 * K,
         "host_library_ms": host_ms, "host_library_threads": pipeline._threads(),
-        "roofline": {"bound": "fp64", "kernel": "calib_kernel", "unit": "TFLOP/s", "peak": FP64_NOMINAL_TFLOPS,
+        "roofline": {"bound": "fp64", "kernel": "moments_kernel + eigen_kernel", "unit": "TFLOP/s", "peak": FP64_NOMINAL_TFLOPS,
                      "peak_kind": "nominal", "fp64_flops_per_call": flops,
                      "achieved": flops / (ms * 1e-3) / 1e12 if flops else None,
                      "frac": flops / (ms * 1e-3) / 1e12 / FP64_NOMINAL_TFLOPS if flops else None},
@@ -574,6 +575,7 @@ def run_measured_leg(args, dev, stream, cals, srcs, cpu_baseline: bool):
 # ---------------------------------------------------------------------------------------
 ROPE_THETA = 500000.0  # Llama-3-8B's rotary base
 ROPE_SOURCES = ["paper_2609_24298_gb300/csrc/rope.cuh", "paper_2609_24298_gb300/csrc/decode.cuh",
+                "paper_2609_24298_gb300/csrc/compress_tc.cuh", "paper_2609_24298_gb300/csrc/compress.cuh",
                 "paper_2609_24298_gb300/csrc/common.cuh"]
 ROPE_PROFILE = os.path.join(ROOT, "profiles", "rope_decode_llama3_8b.txt")
 
@@ -589,7 +591,7 @@ def bf16_peak():
 def run_rope_leg(args, dev, stream, hp, wl, desc, ws, info, q, lens, out, cpu_baseline: bool):
     """Decode attention for a model with the rotary embedding (K compressed before it, Sec. 5
     "Scope"): the same compressed cache, plan and queries as the main step, each key rebuilt,
-    turned to its position and scored (cobra_decode_rope_attn, three launches).  The rebuild is
+    turned to its position and scored (cobra_decode_rope_attn, two launches).  The rebuild is
     a dense contraction, so the leg is measured against the tensor roofline: algorithmic
     FLOPs per call = sum over (seq, layer, kv head) of T (2 d r_K + 2 d G + 2 r_V G).
     Returns the JSON object reported under "rope"."""
@@ -640,13 +642,12 @@ def run_rope_leg(args, dev, stream, hp, wl, desc, ws, info, q, lens, out, cpu_ba
             "unit": "GB/s", "ms_per_call": ms, "calls": K, "theta": ROPE_THETA,
             "workload": f"the main step's cache and queries: {L} layers x {H} kv heads x {S} seqs x {T} tokens, "
                         "query at position T - 1",
-            "roofline": {"bound": "tensor", "kernel": "rope_scan_kernel (timed with its query rotation and "
-                                                      "combine launches)",
+            "roofline": {"bound": "tensor", "kernel": "rope_scan_kernel (timed with its combine launch)",
                          "achieved": achieved, "peak": peak, "peak_kind": kind + " bf16 burst", "unit": "TFLOP/s",
                          "frac": achieved / peak, "algorithmic_flops_per_call": flops,
                          "traffic": profiled_value("traffic_bytes_per_launch", ROPE_PROFILE, ROPE_SOURCES)},
             "cpu_baseline": cpu,
-            "gpu_launches": 3 * K}
+            "gpu_launches": 2 * K}
 
 
 # ---------------------------------------------------------------------------------------

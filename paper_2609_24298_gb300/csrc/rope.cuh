@@ -37,8 +37,8 @@
 // fused multiply-adds).  With 8 warps per SM the latencies between the steps count: X is kept in two
 // halves of 64 columns, so that the next row's MMAs run on the half that has been read while the
 // warps score the other one and accumulate the values.  4 layers x 8 kv heads x 8 x 32768 tokens at
-// 1 bpd: 0.97 ms per call, against 1.80 with the rebuild and the scores on mma.sync (hi + lo of
-// every operand, one warp per row); 1 layer x 8 heads x 8191 tokens at 2 bpd: 36 us, against 390-450
+// 1 bpd: 0.92 to 0.94 ms per call, against 1.80 with the rebuild and the scores on mma.sync (hi + lo of
+// every operand, one warp per row); 1 layer x 8 heads x 8191 tokens at 2 bpd: 33 to 35 us, against 390-450
 // with one CTA per (sequence, layer, kv head).
 #pragma once
 
