@@ -272,7 +272,8 @@ typedef struct {
   long long o_stride_layer, o_stride_seq; /* fp32 elements; query head j at +j*128 */
 } cobra_decode_desc;
 
-/* Workspace bytes for a decode over sequences of at most seq_cap[s] tokens (host [n_seqs]);
+/* Workspace bytes for a decode over sequences of at most seq_cap[s] tokens (host [n_seqs]): the
+ * plan over any capacities up to these, same descriptor and heads otherwise, fits.
  * head_r / head_b: host [>= max params index used] ranks and bit widths of the params. */
 cobra_status cobra_decode_workspace_size(const cobra_decode_desc* desc, const int* head_r, const int* head_b,
                                          const int* seq_cap, size_t* bytes);

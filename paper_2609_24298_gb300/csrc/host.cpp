@@ -873,7 +873,22 @@ struct Plan {
   std::vector<cobra::WsItem> items;
   int max_rv = 0, max_row_bytes = 0;
   int max_stage_bytes = 0;  // largest K channel tiles + V row (128-byte aligned) of a group
+  long long max_items = 0;  // no plan over capacities up to these has more chunks
 };
+
+// Upper bound of the chunks that the plan cuts n_groups groups of `bytes` packed bytes into outside
+// the one-wave calls.  A chunk other than a group's last holds at least 2/3 of its target (the target
+// rounded to whole rows, or one row), and the target f falls with the bytes left, so that together
+// they number at most the integral of 1.5 / f over 0 .. bytes; rising in `bytes`.
+long long guided_items_bound(long long bytes, long long n_groups) {
+  const double lo = (double)kGuide * kScanWarps * kItemMin, hi = (double)kGuide * kScanWarps * kItemMax;
+  const double x = (double)bytes;
+  double n = std::min(x, lo) / kItemMin;
+  if (x > lo) n += (double)kGuide * kScanWarps * std::log(std::min(x, hi) / lo);
+  if (x > hi) n += (x - hi) / kItemMax;
+  // (a target is a whole number of bytes: at most 1 in kItemMin below f)
+  return n_groups + (long long)std::ceil(1.5 * (1.0 + 1.0 / kItemMin) * n);
+}
 
 cobra_status make_plan(const cobra_decode_desc* d, const int* head_r, const int* head_b, const int* seq_cap, Plan& p) {
   cobra_status st = check_decode_desc(d);
@@ -910,18 +925,28 @@ cobra_status make_plan(const cobra_decode_desc* d, const int* head_r, const int*
   };
   long long remaining = 0;  // packed K+V bytes not yet in a chunk
   long long total_rows = 0, total_cost = 0;
+  long long guided_chunks = 0;  // at most, by the limit per group
   size_t max_row = 0;
   for (const Key& k : keys) {
     const long long rows = (seq_cap[k.s] + 127) / 128;
     remaining += rows * pair_bytes(k);
     total_rows += rows;
+    guided_chunks += std::max(1LL, std::min(rows, kMaxChunks));
     total_cost += rows * row_cost(k.rk, k.bk, k.rv, k.bv);
     max_row = std::max(max_row, std::max(cobra_row_bytes(k.rk, k.bk), cobra_row_bytes(k.rv, k.bv)));
   }
   const long long warps = 152LL * cobra::scan_shape(cobra::scan_ring_bytes(max_row), d->group).sm_warps;
   const bool one_wave =
       total_rows <= warps || (total_rows >= kWaveRowsMin * warps && total_rows <= kWaveRowsMax * warps);
-  const long long wave_max = std::min(kWaveMaxChunks, std::max(kMaxChunks, warps / (long long)keys.size()));
+  const long long n_keys = (long long)keys.size();
+  const long long wave_max = std::min(kWaveMaxChunks, std::max(kMaxChunks, warps / n_keys));
+  // Chunks of any plan for these heads whose sequences are as long or shorter.  A shorter call may be
+  // a one-wave call where this one is not: at most a chunk per row, wave_max per group, and warps
+  // chunks besides one per group.  (warps and wave_max do not depend on the lengths.)
+  long long wave_chunks = 0;
+  for (const Key& k : keys) wave_chunks += std::max(1LL, std::min((long long)(seq_cap[k.s] + 127) / 128, wave_max));
+  p.max_items = std::max(std::min(wave_chunks, warps + n_keys),
+                         std::min(guided_chunks, guided_items_bound(remaining, n_keys)));
   for (const Key& key : keys) {
     const int hk = d->k_head0 + key.l * d->layer_stride + key.h, hv = d->v_head0 + key.l * d->layer_stride + key.h;
     p.max_rv = std::max(p.max_rv, key.rv);
@@ -936,7 +961,8 @@ cobra_status make_plan(const cobra_decode_desc* d, const int* head_r, const int*
       g.n_items = 1;
     }
     if (one_wave && rows > 0 && rb > 0) {
-      // rounded down: the chunks of all groups together are at most one per warp
+      // rounded down: the chunks of all groups together are at most one per warp, but for the one that
+      // every group has (more groups than warps)
       const long long share = rows * row_cost(key.rk, key.bk, key.rv, key.bv) * warps / total_cost;
       const long long n = std::max(1LL, std::min(std::min(rows, wave_max), share));
       for (long long c = 0; c < n; ++c) {
@@ -959,7 +985,8 @@ cobra_status make_plan(const cobra_decode_desc* d, const int* head_r, const int*
   return COBRA_OK;
 }
 
-void ws_layout(const cobra_decode_desc* d, const Plan& p, cobra::WsHeader& h, size_t& bytes) {
+// The workspace's layout and size with room for n_items chunks.
+void ws_layout(const cobra_decode_desc* d, const Plan& p, long long n_items, cobra::WsHeader& h, size_t& bytes) {
   std::memset(&h, 0, sizeof(h));
   h.magic = cobra::kWsMagic;
   h.version = COBRA_VERSION;
@@ -978,13 +1005,13 @@ void ws_layout(const cobra_decode_desc* d, const Plan& p, cobra::WsHeader& h, si
   h.groups_off = off = align_up(off, 256);
   off += sizeof(cobra::WsGroup) * p.groups.size();
   h.items_off = off = align_up(off, 256);
-  off += sizeof(cobra::WsItem) * p.items.size();
+  off += sizeof(cobra::WsItem) * (size_t)n_items;
   h.hg_off = off = align_up(off, 256);
   off += sizeof(int32_t) * p.groups.size();
   h.qt_off = off = align_up(off, 256);
   off += (size_t)h.qt_stride * p.groups.size();
   h.part_off = off = align_up(off, 256);
-  off += sizeof(float) * (size_t)h.part_stride * p.items.size();
+  off += sizeof(float) * (size_t)h.part_stride * (size_t)n_items;
   bytes = align_up(off, 256);
 }
 }  // namespace
@@ -996,7 +1023,7 @@ extern "C" cobra_status cobra_decode_workspace_size(const cobra_decode_desc* des
   cobra_status st = make_plan(desc, head_r, head_b, seq_cap, p);
   if (st != COBRA_OK) return st;
   cobra::WsHeader h;
-  ws_layout(desc, p, h, *bytes);
+  ws_layout(desc, p, p.max_items, h, *bytes);
   return COBRA_OK;
 }
 
@@ -1008,7 +1035,7 @@ cobra_status plan_image(const cobra_decode_desc* desc, const int* head_r, const 
   cobra_status st = make_plan(desc, head_r, head_b, seq_cap, p);
   if (st != COBRA_OK) return st;
   cobra::WsHeader h;
-  ws_layout(desc, p, h, *ws_need);
+  ws_layout(desc, p, (long long)p.items.size(), h, *ws_need);
   const size_t head_bytes = h.qt_off;
   img.assign(head_bytes, 0);
   std::memcpy(img.data(), &h, sizeof(h));

@@ -178,3 +178,39 @@ def test_plan_of_one_layer_weighs_the_widths():
     h, g, it, hg = parse(img)
     n1, n2 = g[b[g[:, 5]] == 1, 4], g[b[g[:, 5]] == 2, 4]
     assert n1.min() > 1.2 * n2.max() and g[:, 4].sum() <= 152 * 16
+
+
+def plan_bytes(desc, r, b, caps):
+    """Bytes of the workspace that a plan over `caps` uses."""
+    img, info = cobra.cobra_decode_plan_host(desc, r, b, caps)
+    h, *_ = parse(img)
+    return (h["part_off"] + 4 * h["part_stride"] * h["n_items"] + 255) // 256 * 256
+
+
+@pytest.mark.parametrize("L,H,S,G,rb,T", [
+    (1, 8, 1, 4, (64, 2), 131072),   # a shorter call is cut in one wave of more chunks
+    (1, 8, 1, 8, (64, 2), 131072),
+    (1, 1, 3, 4, (30, 1), 65536),
+    (2, 4, 24, 4, None, 6001),
+    (32, 8, 8, 4, None, 32768),
+    (1, 8, 6, 8, (126, 8), 40000),
+    (16, 8, 5, 8, None, 3000),
+])
+def test_workspace_size_covers_every_shorter_call(L, H, S, G, rb, T):
+    """A workspace sized for the longest sequences has room for the plan over any shorter ones."""
+    rng = np.random.default_rng(L + S + T)
+    n = 2 * L * H
+    r = np.full(n, rb[0], np.int32) if rb else (2 * rng.integers(0, 65, n)).astype(np.int32)
+    b = np.full(n, rb[1], np.int32) if rb else rng.integers(1, 9, n).astype(np.int32)
+    d = cobra.decode_desc(k_head0=0, v_head0=L * H, layer_stride=H, n_layers=L, n_kv_heads=H, group=G, n_seqs=S,
+                          rows_per_seq=(T + 127) // 128, pages_per_seq=0)
+    caps = np.full(S, T)
+    size = cobra.cobra_decode_workspace_size(d, r, b, caps)
+    assert plan_bytes(d, r, b, caps) <= size
+    shorter = [np.full(S, max(1, int(T * f))) for f in np.geomspace(1 / T, 1, 40)]
+    shorter += [np.minimum(T, np.exp(rng.uniform(0, np.log(T), S)).astype(int)) for _ in range(40)]
+    shorter += [np.where(np.arange(S) == 0, T, 0)]
+    for c in shorter:
+        assert plan_bytes(d, r, b, c) <= size
+        # (and a size asked for the shorter call is no larger either)
+        assert cobra.cobra_decode_workspace_size(d, r, b, c) <= size
