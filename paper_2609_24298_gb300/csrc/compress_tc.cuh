@@ -355,18 +355,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int head_local = blockIdx.x / a.chunks, chunk = blockIdx.x % a.chunks;
   const int layer = head_local / a.n_kv, kv = head_local % a.n_kv;
-  const HeadEntry he = head_table(a.block)[a.head0 + layer * a.layer_stride + kv];
-  const int r = he.r, b = he.b;
   const int nrows = (a.n_tok + kRowTokens - 1) / kRowTokens;
   const int ntiles = a.n_seqs * nrows;
   grid_dep_launch();
-  if (r == 0 || chunk >= ntiles) {
+  if (chunk >= ntiles) {
     grid_dep_wait();
     return;
   }
   const int my_tiles = (ntiles - chunk + a.chunks - 1) / a.chunks;
-  const int nsplit = b >= 6 ? 3 : 2;
-  const float* pool = param_pool(a.block);
   const uint32_t bar0 = smem_addr(bars);
   auto bar = [&](int i) { return bar0 + 8u * i; };
   const int XF = 0, XE = kTcStages, AF = 2 * kTcStages, AE = AF + 2, DONE = AF + 4, WREADY = AF + 5;
@@ -392,9 +388,18 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_holder;
 
-  if (warp == 0) {
+  // Only the setup above overlaps the kernel ahead: the parameter block and X may be its results,
+  // and it may still read the cache rows written below.
+  grid_dep_wait();
+  const HeadEntry he = head_table(a.block)[a.head0 + layer * a.layer_stride + kv];
+  const int r = he.r, b = he.b;
+  const int nsplit = b >= 6 ? 3 : 2;
+  const float* pool = param_pool(a.block);
+
+  if (r == 0) {
+    // no code rows
+  } else if (warp == 0) {
     // ---------------- TMA producer ----------------
-    grid_dep_wait();  // X may be the result of a kernel ahead
     if (lane == 0) {
       int issued = 0;
       for (int i = 0; i < my_tiles; ++i) {
@@ -424,7 +429,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: Y^T[128 channels][128 tokens] per tile ----------------
-    grid_dep_wait();
     if (lane == 0) {
       const uint32_t idesc = umma_idesc_bf16(128, 128);
       const uint32_t xbase = smem_addr(xsm);
@@ -503,7 +507,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(WREADY));
     }
-    grid_dep_wait();  // kernels ahead may still read the cache rows written below
     TcEpi e;
     const float scale = 1.0f / (float)(1 << b);  // a power of two: the scaled values are exact
     e.inv_s = he.inv_delta * scale;

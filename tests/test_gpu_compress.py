@@ -217,3 +217,31 @@ def test_few_tiles_spread_over_ctas(H, S, T):
                 rb = 16 * int(r[h]) * int(b[h])
                 a = host[int(offs[h]) + q * rows * rb:][:rows * rb]
                 assert np.array_equal(a, one[int(o1[h]):][:rows * rb])
+
+
+def test_parameters_written_by_the_kernel_ahead():
+    """Stream order covers the parameter block: the kernel directly ahead writes a head's basis (here
+    the angle table's kernel, whose 16 + 112 rows of 128 floats are a basis of rank 128), and the
+    codes are those of the finished block."""
+    T, r, b = 640, 128, 2
+    g = np.random.default_rng(5)
+    x = torch.tensor(g.standard_normal((T, 128)), dtype=torch.bfloat16, device=DEV)
+    p = dict(r=r, b=b, W=np.eye(128, dtype=np.float32), mu=np.zeros(128, np.float32), delta=np.float32(4.0))
+    nrows = T // 128
+    block, offs, total, rr, bb = upload([p], nrows)
+    w_ptr = block.data_ptr() + 256  # header, one head entry, pool at the next multiple of 256 bytes
+    desc = cobra.compress_desc(head0=0, layer_stride=1, n_layers=1, n_kv_heads=1, side=0, n_seqs=1, rows_per_seq=nrows,
+                               pages_per_seq=0, x_stride_layer=0, x_stride_seq=T * 128, x_stride_tok=128, x_stride_head=128)
+    got = []
+    for theta in (3.0, 500000.0, 3.0):
+        cache = torch.zeros(total, dtype=torch.uint8, device=DEV)
+        torch.cuda.synchronize()
+        cobra.cobra_rope_table(theta, 16 * 112, w_ptr, 128 * 128 * 4)
+        cobra.cobra_compress(block, desc, x, 0, T, cache, None)  # directly behind
+        again = torch.zeros_like(cache)
+        torch.cuda.synchronize()
+        cobra.cobra_compress(block, desc, x, 0, T, again, None)
+        assert cobra.cobra_check() == cobra.COBRA_OK
+        assert torch.equal(cache, again)
+        got.append(cache)
+    assert torch.equal(got[0], got[2]) and not torch.equal(got[0], got[1])
