@@ -29,7 +29,6 @@
 
 namespace cobra {
 
-constexpr int kDecodeWarps = 4;  // per CTA at most (see scan_shape)
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s
 
 struct DecodeArgs {
@@ -543,7 +542,7 @@ __device__ __forceinline__ void scan_item(const DecodeArgs& a, ScanWarp& w, int 
 }
 
 template <int G>
-__global__ void __launch_bounds__(kDecodeWarps * 32, G == 4 ? 4 : 3) decode_kernel(DecodeArgs a) {
+__global__ void __launch_bounds__(kScanCtaWarps * 32, scan_reg_warps(G) / kScanCtaWarps) decode_kernel(DecodeArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   // the combine kernel may be scheduled as CTAs of this grid exit (it waits for the results)
   grid_dep_launch();

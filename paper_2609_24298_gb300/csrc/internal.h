@@ -87,20 +87,26 @@ constexpr size_t scan_ring_bytes(size_t max_row) {
 // The scan's shared memory per warp besides the ring: V accumulators and query fragments.
 constexpr size_t scan_state_bytes(int group) { return group == 4 ? 4352 : 8704; }
 
-// Warps per scan CTA and resident warps per SM (at most 16, the registers' limit): 4, 2 or 1 warps,
+// Resident scan warps per SM that the registers allow: 128 a thread with 4 query heads per kv head, 168
+// with 8 (the scan's launch bounds are made of these).
+constexpr int kScanCtaWarps = 4;  // per CTA at most
+constexpr int scan_reg_warps(int group) { return group == 4 ? 16 : 12; }
+
+// Warps per scan CTA and resident warps per SM (at most what the registers allow): 4, 2 or 1 warps,
 // whichever fits the most into 228 KB of shared memory (1 KB of it per CTA is the system's); the
 // larger CTA of equals, whose launches are fewer.  A layer of 8 kv heads x 8 x 32768 tokens at 1 bpd
 // (8 KB rings) takes 57 us per step with 4, 60 with 2 and 65 with 1; 2 layers x 32 ragged sequences at
-// 4 bpd (24 to 32 KB rings) 639, 547 and 541.
+// 4 bpd (24 to 32 KB rings) 639, 547 and 541.  With 8 query heads the layer takes 67 us; 76 in CTAs of
+// one warp and chunks for the 13 warps per SM that shared memory alone would hold.
 struct ScanShape {
   int cta_warps, sm_warps;
 };
 constexpr ScanShape scan_shape(size_t ring, int group) {
   ScanShape best{1, 0};
-  for (int nw = 4; nw >= 1; nw /= 2) {
+  for (int nw = kScanCtaWarps; nw >= 1; nw /= 2) {
     const size_t cta = nw * (ring + scan_state_bytes(group)) + 1024;
-    const size_t n = nw * (233472 / cta);
-    const int warps = n < 16 ? (int)n : 16;
+    const int n = (int)(233472 / cta) * nw, limit = scan_reg_warps(group) / nw * nw;
+    const int warps = n < limit ? n : limit;
     if (warps > best.sm_warps) best = ScanShape{nw, warps};
   }
   return best;

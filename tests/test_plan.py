@@ -143,17 +143,21 @@ def test_plan_host_reports_size_without_buffer():
         cobra.cobra_decode_plan_host(d, r, b, [4096])  # beyond rows_per_seq
 
 
-@pytest.mark.parametrize("S,T,rb,rows_per_chunk", [
-    (1, 2048, (128, 2), (1, 1)),       # fewer rows than warps: a warp per row
-    (8, 32768, (64, 2), (6, 8)),       # a layer of long sequences: one chunk per warp
-    (8, 32768, (64, 3), (6, 8)),
-    (3, 131072, (64, 2), (16, 17)),    # few groups: at most 64 chunks each
-    (24, 2944, (64, 3), None),         # between the two: chunks of at least 16 KB, taken as warps free up
+@pytest.mark.parametrize("S,T,rb,rows_per_chunk,G", [
+    (1, 2048, (128, 2), (1, 1), 4),       # fewer rows than warps: a warp per row
+    (8, 32768, (64, 2), (6, 8), 4),       # a layer of long sequences: one chunk per warp
+    (8, 32768, (64, 3), (6, 8), 4),
+    (3, 131072, (64, 2), (16, 17), 4),    # few groups: at most 64 chunks each
+    (24, 2944, (64, 3), None, 4),         # between the two: chunks of at least 16 KB, taken as warps free up
+    (6, 32768, (64, 2), (6, 8), 8),       # 8 query heads: 12 warps per SM
+    (8, 32768, (64, 2), (8, 10), 8),
+    (8, 32768, (128, 2), (8, 10), 8),
+    (5, 32768, (128, 4), (8, 11), 8),     # 16 KB rings: 8 warps per SM
 ])
-def test_plan_of_one_layer_fills_one_wave(S, T, rb, rows_per_chunk):
+def test_plan_of_one_layer_fills_one_wave(S, T, rb, rows_per_chunk, G):
     H = 8
     r, b = np.full(2 * H, rb[0], np.int32), np.full(2 * H, rb[1], np.int32)
-    d, img, info = make(1, H, S, [T] * S, r, b)
+    d, img, info = make(1, H, S, [T] * S, r, b, G)
     h, g, it, hg = parse(img)
     rows = T // 128
     for gi, (s, l, kv, first, n, hk, hv, _) in enumerate(g):
@@ -164,7 +168,11 @@ def test_plan_of_one_layer_fills_one_wave(S, T, rb, rows_per_chunk):
     size = it[:, 2] - it[:, 1]
     if rows_per_chunk:
         assert size.min() >= rows_per_chunk[0] and size.max() <= rows_per_chunk[1]
-        assert len(it) <= 152 * 16 and g[:, 4].max() <= 64
+        # resident scan warps: 16 or 12 per SM by their registers, or what fits 228 KB of shared memory
+        # (a CTA: the rings, 4352 or 8704 bytes of state per warp, 1 KB of the system's)
+        ring, state = max(8192, 2 * 16 * rb[0] * rb[1]), 4352 if G == 4 else 8704
+        fit = max(min(16 if G == 4 else 12, nw * (233472 // (nw * (ring + state) + 1024))) for nw in (4, 2, 1))
+        assert len(it) <= 152 * fit and g[:, 4].max() <= 64
     else:
         assert size.min() >= 1 and len(it) > 152 * 8
 
