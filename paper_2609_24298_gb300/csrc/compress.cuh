@@ -152,7 +152,7 @@ __device__ __forceinline__ void proj_unit(const ProjSmem& sm, int vg, int cb, in
 }
 // Os <- projections of the nv vectors in Xs on the r channels.  Wider units read each basis value
 // for more vectors' worth of work per shared-memory access; they are used once there are enough
-// of them for the 8 warps.
+// of them for the 8 warps, and no wider than the head's channels.
 template <int CB>
 __device__ __forceinline__ void proj_units(const ProjSmem& sm, int nv, int r) {
   const int ng = (nv + 3) >> 2, nc = ((r + 31) / 32 + CB - 1) / CB;
@@ -162,7 +162,7 @@ __device__ __forceinline__ void project(const ProjSmem& sm, int nv, int r) {
   const int units = ((nv + 3) >> 2) * ((r + 31) / 32);
   if (units <= kProjWarps)
     proj_units<1>(sm, nv, r);
-  else if (units <= 2 * kProjWarps)
+  else if (units <= 2 * kProjWarps || r <= 64)
     proj_units<2>(sm, nv, r);
   else
     proj_units<4>(sm, nv, r);

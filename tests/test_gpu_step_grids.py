@@ -74,14 +74,14 @@ def test_alignment_of_tokens_and_queries(heads, S, G):
         assert np.array_equal(c0, c1) and np.array_equal(o0, o1)
 
 
-@pytest.mark.parametrize("S", [5, 11])
-def test_one_cta_per_head_equals_split_heads(heads, S):
-    """80 layers x 2 heads fill the GPU (one CTA per head, two passes at 11 sequences); a layer
-    alone spreads its heads' sequences over CTAs."""
+@pytest.mark.parametrize("S,G", [(5, 4), (7, 4), (11, 4), (15, 4), (7, 8)])
+def test_one_cta_per_head_equals_split_heads(heads, S, G):
+    """80 layers x 2 heads fill the GPU (one CTA per head: passes of 8 sequences and a rest, of 7 with
+    a warp left over, of 4 with 8 query heads); a layer alone spreads its heads' sequences over CTAs."""
     layers = 80
-    c0, o0, offs, n_slots, r, b = step(heads, layers, S, 4)
+    c0, o0, offs, n_slots, r, b = step(heads, layers, S, G)
     for layer in (0, 37, 79):
-        c1, o1, *_ = step(heads, layers, S, 4, layer=layer)
+        c1, o1, *_ = step(heads, layers, S, G, layer=layer)
         for h in (2 * layer, 2 * layer + 1, 2 * (layers + layer), 2 * (layers + layer) + 1):
             at = slice(int(offs[h]), int(offs[h]) + n_slots * 16 * int(r[h]) * int(b[h]))
             assert np.array_equal(c0[at], c1[at])
