@@ -14,8 +14,8 @@ namespace cobra {
 // ---------------------------------------------------------------------------------------
 // Per-head kernels: the query projection has one CTA of 256 threads per (layer, kv head) and run
 // of sequences, 32 query vectors per pass, with the head's basis staged in shared memory once; the
-// combine has one per (layer, kv head, sequence).  The workspace's head-group table gives the group
-// of (head, seq).
+// combine has one per (layer, kv head) and one or two sequences.  The workspace's head-group table
+// gives the group of (head, seq).
 // ---------------------------------------------------------------------------------------
 constexpr int kHeadThreads = 256;
 constexpr int kVecPass = 32;  // query vectors (sequences x G) per pass
@@ -208,30 +208,38 @@ __global__ void __launch_bounds__(kHeadThreads, 2) qproj_kernel(DecodeArgs a, Co
 //   per query head: m* = max over chunks, l* = sum 2^(m - m*) l, zbar = Delta_V (sum 2^(m - m*)
 //   acc / l* - 2^{b-1} + 1/2), o = mu_V + W_V zbar (zeros for an empty sequence).
 //
-// One CTA of 256 threads per (layer, kv head, sequence).  The kernel is a chain of memory round
-// trips (chunk maxima, chunk sums, the rows of W_V), so every phase spreads its loads over all
-// threads and issues them together; a head's W_V is read again for each sequence (from L2).
+// One CTA of 256 threads per (layer, kv head) and run of NS sequences.  The kernel is a chain of
+// memory round trips (chunk maxima, chunk sums, the rows of W_V), so every phase spreads its loads
+// over all threads and issues them together; a head's W_V is read again for each run (from L2).
 // Against one CTA per head and run of 16 query vectors, a step over 1 layer x 8 kv heads takes
 // 23 us for 25.9 (1 x 2048 tokens), 50 for 67 (24 ragged sequences at 3 bpd) and 63 for 80
-// (8 x 32768); over all 32 layers it takes the same 876 us.
+// (8 x 32768).  NS = 1 spreads a call over the most CTAs; with 4 query heads, calls that would take
+// more than two rounds of resident CTAs share W_V between two sequences where that takes fewer rounds
+// (combine_seqs): 32 layers x 8 heads x 16 sequences 33.5 us for 46.5 with NS = 1, x 64 sequences 125 for
+// 187 (112 with runs of 16 vectors); 1 layer x 64 sequences would take 8.6 for 8.5, its step 45.7 for 44.2.
 // ---------------------------------------------------------------------------------------
-template <int G>
-__global__ void __launch_bounds__(kHeadThreads, 3) combine_kernel(DecodeArgs a) {
-  __shared__ float wts[G][kWtChunk];          // weights 2^(m_k - m*) / l* of a round of chunks
-  __shared__ float m_s[G], inv_l_s[G];
-  __shared__ __align__(16) float red[kHeadThreads * 4];  // partial chunk sums, then zbar [channel][G]
+constexpr int kCombineCtas = 3;  // resident per SM
+template <int G, int NS>
+__global__ void __launch_bounds__(kHeadThreads, kCombineCtas) combine_kernel(DecodeArgs a) {
+  constexpr int V = G * NS;  // query vectors of the CTA: vector v = query head v % G of sequence s0 + v / G
+  static_assert(V <= kHeadThreads / 32, "a warp per vector");
+  __shared__ float wts[V][kWtChunk];          // weights 2^(m_k - m*) / l* of a round of chunks
+  __shared__ float m_s[V], inv_l_s[V];
+  __shared__ __align__(16) float red[kHeadThreads * 4];  // partial chunk sums, then zbar [channel][V]
   const WsHeader* wh = reinterpret_cast<const WsHeader*>(a.ws);
   const WsGroup* groups = reinterpret_cast<const WsGroup*>(a.ws + wh->groups_off);
   const float* parts = reinterpret_cast<const float*>(a.ws + wh->part_off);
   const int S = wh->n_seqs, pstride = wh->part_stride, gstride = wh->g_stride;
-  const WsGroup gr = groups[reinterpret_cast<const int*>(a.ws + wh->hg_off)[blockIdx.x]];
-  const HeadEntry hv = head_table(a.block)[gr.v_head];
+  const int runs = (S + NS - 1) / NS, s0 = (int)(blockIdx.x % runs) * NS;
+  const int* hg = reinterpret_cast<const int*>(a.ws + wh->hg_off) + (size_t)(blockIdx.x / runs) * S;
+  const WsGroup g0 = groups[hg[s0]], g1 = groups[hg[min(s0 + NS, S) - 1]];  // (NS <= 2)
+  const HeadEntry hv = head_table(a.block)[g0.v_head];
   const float* pool = param_pool(a.block);
   const int rv = hv.r, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const float* W = pool + hv.w_off;
   // W_V is pulled into L2 here, while the scan ahead of this kernel is still finishing (the first
-  // sequence's CTA of a head does it for all)
-  if (blockIdx.x % S == 0)
+  // run's CTA of a head does it for all)
+  if (s0 == 0)
     for (int idx = tid; idx < rv * (kD / 32); idx += kHeadThreads) prefetch_l2(W + 32 * idx);
   const int d0 = 16 * warp + 4 * (lane & 3);  // dims of the back-projection: d0 .. d0 + 3
   const float4 mu4 = *reinterpret_cast<const float4*>(pool + hv.mu_off + d0);
@@ -239,13 +247,19 @@ __global__ void __launch_bounds__(kHeadThreads, 3) combine_kernel(DecodeArgs a) 
   grid_dep_launch();
   // everything above is independent of the scan; its partials are read only from here on
   grid_dep_wait();
-  const int n = a.seq_lens[gr.seq] > 0 ? gr.n_items : 0;
-  const float* part = parts + (size_t)gr.first_item * pstride;
-  // (1) warp g: m* and l* of query head g, lanes over chunks, merged online (a chunk with no tokens
+  const int n0 = a.seq_lens[g0.seq] > 0 ? g0.n_items : 0;
+  const int n1 = NS > 1 && s0 + 1 < S && a.seq_lens[g1.seq] > 0 ? g1.n_items : 0, nmax = max(n0, n1);
+  // chunks of a vector's sequence, and the first one's partial
+  auto chunks = [&](int v) { return NS == 1 || v < G ? n0 : n1; };
+  auto first = [&](int v) {
+    return parts + (size_t)(NS == 1 || v < G ? g0 : g1).first_item * pstride + (v % G) * gstride;
+  };
+  // (1) warp v: m* and l* of vector v, lanes over chunks, merged online (a chunk with no tokens
   //     has m = -inf and no value entries; its weight is zero).  The m of the first kWtChunk chunks
   //     stay in shared memory and become the weights of the first round of (2).
-  if (warp < G) {
-    const float* pg = part + warp * gstride;
+  if (warp < V) {
+    const float* pg = first(warp);
+    const int n = chunks(warp);
     float M = -INFINITY, Ls = 0.f;
     for (int k = lane; k < n; k += 32) {
       const float mk = pg[(size_t)k * pstride], lk = pg[(size_t)k * pstride + 1];
@@ -276,31 +290,31 @@ __global__ void __launch_bounds__(kHeadThreads, 3) combine_kernel(DecodeArgs a) 
     }
   }
   __syncthreads();
-  // (2) weighted chunk sums: thread (channel quad cq, query head g, chunk share p) of rw = r_V
+  // (2) weighted chunk sums: thread (channel quad cq, vector v, chunk share p) of rw = r_V
   //     rounded up to 32, 64 or 128 channels sums 16-byte entries of chunks p, p + np, ..., eight
   //     loads in flight; the shares are added through shared memory.
   const int rw = rv <= 32 ? 32 : rv <= 64 ? 64 : kD;
-  const int nq = rw / 4, np = kHeadThreads / (nq * G);  // np >= 1 (G = 8, rw = 128)
+  const int nq = rw / 4, np = kHeadThreads / (nq * V);  // np >= 1 (V = 8, rw = 128)
   {
-    const int cq = tid % nq, g = (tid / nq) % G, p = tid / (nq * G);
+    const int cq = tid % nq, v = (tid / nq) % V, p = tid / (nq * V), n = chunks(v);
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int k0 = 0; k0 < n; k0 += kWtChunk) {
+    for (int k0 = 0; k0 < nmax; k0 += kWtChunk) {
       if (k0 > 0) {  // later rounds: one weight per thread into shared memory
         __syncthreads();
-        for (int idx = tid; idx < G * kWtChunk; idx += kHeadThreads) {
-          const int v = idx / kWtChunk, k = k0 + idx % kWtChunk;
+        for (int idx = tid; idx < V * kWtChunk; idx += kHeadThreads) {
+          const int vw = idx / kWtChunk, k = k0 + idx % kWtChunk;
           float w = 0.f;
-          if (k < n) {
-            const float mk = part[(size_t)k * pstride + v * gstride];
-            if (mk != -INFINITY) w = exp2f(mk - m_s[v]) * inv_l_s[v];
+          if (k < chunks(vw)) {
+            const float mk = first(vw)[(size_t)k * pstride];
+            if (mk != -INFINITY) w = exp2f(mk - m_s[vw]) * inv_l_s[vw];
           }
-          wts[v][idx % kWtChunk] = w;
+          wts[vw][idx % kWtChunk] = w;
         }
         __syncthreads();
       }
       if (4 * cq >= rv) continue;
       // the partial's channels start 4 floats in and every stride is a multiple of 4 floats
-      const float4* px = reinterpret_cast<const float4*>(part + (size_t)k0 * pstride + g * gstride + 4 + 4 * cq);
+      const float4* px = reinterpret_cast<const float4*>(first(v) + (size_t)k0 * pstride + 4 + 4 * cq);
       const int kr = min(kWtChunk, n - k0);
       for (int kb = p; kb < kr; kb += 8 * np) {
         float4 x[8];
@@ -308,7 +322,7 @@ __global__ void __launch_bounds__(kHeadThreads, 3) combine_kernel(DecodeArgs a) 
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           const int k = kb + u * np;
-          w[u] = k < kr ? wts[g][k] : 0.f;
+          w[u] = k < kr ? wts[v][k] : 0.f;
           // an empty chunk's value entries were never written
           x[u] = w[u] != 0.f ? px[(size_t)k * (pstride / 4)] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
@@ -324,32 +338,32 @@ __global__ void __launch_bounds__(kHeadThreads, 3) combine_kernel(DecodeArgs a) 
     *reinterpret_cast<float4*>(red + 4 * tid) = acc;
   }
   __syncthreads();
-  // zbar = Delta (sum_k w_k acc_k - 2^{b-1} + 1/2), written back as [channel][G]
+  // zbar = Delta (sum_k w_k acc_k - 2^{b-1} + 1/2), written back as [channel][V]
   {
     const float cen = rv > 0 ? (float)(1 << (hv.b - 1)) - 0.5f : 0.f;
-    float z[G / 2];  // at most G rw / 256 <= G / 2 values per thread
+    float z[V / 2];  // at most V rw / 256 <= V / 2 values per thread
 #pragma unroll
-    for (int u = 0; u < G / 2; ++u) {
-      const int idx = tid + u * kHeadThreads;  // g rw + channel
+    for (int u = 0; u < V / 2; ++u) {
+      const int idx = tid + u * kHeadThreads;  // v rw + channel
       float sum = 0.f;
-      if (idx < G * rw)
-        for (int p = 0; p < np; ++p) sum += red[p * G * rw + idx];
-      z[u] = n > 0 ? hv.delta * (sum - cen) : 0.f;
+      if (idx < V * rw)
+        for (int p = 0; p < np; ++p) sum += red[p * V * rw + idx];
+      z[u] = chunks(idx / rw) > 0 ? hv.delta * (sum - cen) : 0.f;
     }
     __syncthreads();
 #pragma unroll
-    for (int u = 0; u < G / 2; ++u) {
+    for (int u = 0; u < V / 2; ++u) {
       const int idx = tid + u * kHeadThreads;
-      if (idx < G * rw) red[(idx % rw) * G + idx / rw] = z[u];
+      if (idx < V * rw) red[(idx % rw) * V + idx / rw] = z[u];
     }
   }
   __syncthreads();
   // (3) o = mu_V + W_V zbar: a warp has 16 dims, its lanes 4 dims x every eighth row of W_V (eight
   //     16-byte loads in flight); the eight row shares are added by halving exchanges, after which
-  //     a lane holds G / 2 consecutive outputs.
-  float o[4 * G];
+  //     a lane holds V / 2 consecutive outputs.
+  float o[4 * V];
 #pragma unroll
-  for (int k = 0; k < 4 * G; ++k) o[k] = 0.f;
+  for (int k = 0; k < 4 * V; ++k) o[k] = 0.f;
   const int sl = lane >> 2;
   const float4* W4 = reinterpret_cast<const float4*>(W + d0);
   for (int i0 = sl; i0 < rv; i0 += 64) {
@@ -360,37 +374,39 @@ __global__ void __launch_bounds__(kHeadThreads, 3) combine_kernel(DecodeArgs a) 
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       // rows past r_V have w = 0; their zbar is finite (zeros, or within rw <= 128 rows)
-      const float* zr = red + (i0 + 8 * u < rv ? i0 + 8 * u : 0) * G;
+      const float* zr = red + (i0 + 8 * u < rv ? i0 + 8 * u : 0) * V;
 #pragma unroll
-      for (int g = 0; g < G; ++g) {
-        const float zz = zr[g];
-        o[4 * g + 0] += w[u].x * zz;
-        o[4 * g + 1] += w[u].y * zz;
-        o[4 * g + 2] += w[u].z * zz;
-        o[4 * g + 3] += w[u].w * zz;
+      for (int v = 0; v < V; ++v) {
+        const float zz = zr[v];
+        o[4 * v + 0] += w[u].x * zz;
+        o[4 * v + 1] += w[u].y * zz;
+        o[4 * v + 2] += w[u].z * zz;
+        o[4 * v + 3] += w[u].w * zz;
       }
     }
   }
 #pragma unroll
   for (int st = 0; st < 3; ++st) {
-    const int half = (4 * G) >> (st + 1), bit = 16 >> st;
+    const int half = (4 * V) >> (st + 1), bit = 16 >> st;
     const bool up = lane & bit;
 #pragma unroll
-    for (int k = 0; k < (4 * G) >> 1; ++k) {
+    for (int k = 0; k < (4 * V) >> 1; ++k) {
       if (k < half) {
         const float send = up ? o[k] : o[half + k], keep = up ? o[half + k] : o[k];
         o[k] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
       }
     }
   }
-  // lane share sl holds outputs [sl G / 2, (sl + 1) G / 2) of the 4 G (query head, dim) values
+  // lane share sl holds outputs [sl V / 2, (sl + 1) V / 2) of the 4 V (vector, dim) values
   const float mu_a[4] = {mu4.x, mu4.y, mu4.z, mu4.w};
 #pragma unroll
-  for (int k = 0; k < G / 2; ++k) {
-    const int e = sl * (G / 2) + k, g = e >> 2, c = e & 3;
-    const float mu = (G == 8) ? mu_a[k & 3] : ((sl & 1) ? mu_a[2 + k] : mu_a[k]);
+  for (int k = 0; k < V / 2; ++k) {
+    const int e = sl * (V / 2) + k, v = e >> 2, c = e & 3;
+    const WsGroup& gr = NS == 1 || v < G ? g0 : g1;
+    if (NS > 1 && v >= G && s0 + 1 >= S) break;
+    const float mu = (V == 8) ? mu_a[k & 3] : ((sl & 1) ? mu_a[2 + k] : mu_a[k]);
     // the output is only 4-byte aligned in general
-    a.out[gr.layer * a.o_sl + gr.seq * a.o_ss + (long long)(gr.kv * G + g) * kD + d0 + c] = n > 0 ? mu + o[k] : 0.f;
+    a.out[gr.layer * a.o_sl + gr.seq * a.o_ss + (long long)(gr.kv * G + v % G) * kD + d0 + c] = chunks(v) > 0 ? mu + o[k] : 0.f;
   }
 }
 

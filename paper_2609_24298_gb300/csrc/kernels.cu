@@ -231,6 +231,15 @@ ProjSplit proj_split(long long heads, int n_seqs) {
   return {(n_seqs + spb - 1) / spb, spb};
 }
 
+// Sequences per combine CTA: two where that is fewer rounds of resident CTAs, by more than a CTA of
+// two sequences takes longer (5.1 against 6.5 us per round), and the call has more than two rounds
+// (kernels of one or two rounds hide behind the scan's tail; NS = 1 starts sooner).
+int combine_seqs(int group, long long n_heads, int n_seqs) {
+  const long long resident = (long long)kCombineCtas * sm_count();
+  auto rounds = [&](int ns) { return (n_heads * ((n_seqs + ns - 1) / ns) + resident - 1) / resident; };
+  return group == 4 && rounds(1) > 2 && 3 * rounds(1) > 4 * rounds(2) ? 2 : 1;
+}
+
 // validated append arguments for one side
 cobra_status append_args(const void* params, const cobra_compress_desc* d, const void* x, const int* pos,
                          uint8_t* cache, const int* page_table, CompressArgs& a) {
@@ -316,11 +325,13 @@ cobra_status launch_decode(const DecodeArgs& a, int n_heads, int n_seqs, int n_i
     if (launch_pdl(decode_kernel<G>, (unsigned)grid, (unsigned)(nw * 32), smem, s, a) != cudaSuccess) return COBRA_ECUDA;
   }
   if (stages & kCombine) {
-    // one CTA per (layer, kv head, sequence); its prologue (the plan, the L2 prefetch of W_V)
-    // overlaps the scan's tail
-    const long long grid = (long long)n_heads * n_seqs;
+    // its prologue (the plan, the L2 prefetch of W_V) overlaps the scan's tail
+    const int ns = combine_seqs(G, n_heads, n_seqs);
+    const long long grid = (long long)n_heads * ((n_seqs + ns - 1) / ns);
     if (grid > 0x7fffffffLL) return COBRA_EINVAL;
-    if (launch_pdl(combine_kernel<G>, (unsigned)grid, kHeadThreads, 0, s, a) != cudaSuccess) return COBRA_ECUDA;
+    if (launch_pdl(ns == 2 ? combine_kernel<G, 8 / G> : combine_kernel<G, 1>, (unsigned)grid, kHeadThreads, 0, s, a) !=
+        cudaSuccess)
+      return COBRA_ECUDA;
   }
   return COBRA_OK;
 }

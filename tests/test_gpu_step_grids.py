@@ -27,10 +27,10 @@ def heads():
     return [oracle_head(s, r, b) for s, (r, b) in zip(srcs, [(128, 2), (34, 5), (100, 1), (64, 3)])]
 
 
-def step(heads, layers, S, G, layer=None, shift=0, paged=False, cap=256):
+def step(heads, layers, S, G, layer=None, shift=0, paged=False, cap=256, empty=None):
     """One step over `layers` copies of the two heads (or over layer `layer` alone) on a cache of
     constant bytes; inputs are the same whatever the form.  shift: elements the inputs are moved
-    from their 16-byte boundary."""
+    from their 16-byte boundary; empty: a sequence whose length reads 0 in the attention."""
     n = 2 * layers
     params = heads[:2] * layers + heads[2:] * layers
     n_slots = S * ROWS
@@ -60,6 +60,8 @@ def step(heads, layers, S, G, layer=None, shift=0, paged=False, cap=256):
     info = cobra.cobra_decode_plan(desc, r, b, lens, ws, wsb)
     out = torch.full((L, S, 2 * G, 128), float("nan"), dtype=torch.float32, device=DEV)
     ld, pos = torch.tensor(lens, device=DEV), torch.tensor(lens - 1, device=DEV)
+    if empty is not None:
+        ld[empty] = 0
     cobra.cobra_decode_step(block, desc, info, side(0), side(1), kp, vp, pos, qp, cache, ld, None, out, ws, wsb)
     assert cobra.cobra_check() == cobra.COBRA_OK
     return cache.cpu().numpy(), out.cpu().numpy(), offs, n_slots, r, b
@@ -86,3 +88,17 @@ def test_one_cta_per_head_equals_split_heads(heads, S, G):
             at = slice(int(offs[h]), int(offs[h]) + n_slots * 16 * int(r[h]) * int(b[h]))
             assert np.array_equal(c0[at], c1[at])
         assert rel_err(o1[0], o0[layer]) < 2e-3  # the chunks of the two plans differ
+
+
+@pytest.mark.parametrize("S,empty", [(6, None), (7, None), (7, 0)])
+def test_combine_of_two_sequences_per_cta(heads, S, empty):
+    """80 layers x 2 heads x 6 or 7 sequences of one chunk each are combined two sequences to a CTA
+    (the last one alone when S is odd), a layer alone one to a CTA: the same partials, the same
+    outputs.  An empty sequence gives zeros in either."""
+    layers = 80
+    _, o0, *_ = step(heads, layers, S, 4, cap=128, empty=empty)
+    for layer in (0, 37, 79):
+        _, o1, *_ = step(heads, layers, S, 4, layer=layer, cap=128, empty=empty)
+        assert np.array_equal(o1[0], o0[layer])
+    if empty is not None:
+        assert np.all(o0[:, empty] == 0) and np.all(o0[:, empty + 1] != 0)
