@@ -662,7 +662,6 @@ __global__ void __launch_bounds__(MAXWG * 160, 1) rope_scan_kernel(DecodeArgs a,
               }
             }
           }
-          if (expired) atomicOr(&g_status, 1u);
           // the last V rows of a single stage: row n - 1's is free once row n's scores are in, which the
           // second half's last read tells
           if (rbv && ns == 1 && n_rows >= 2 && !expired) {
@@ -670,9 +669,10 @@ __global__ void __launch_bounds__(MAXWG * 160, 1) rope_scan_kernel(DecodeArgs a,
               fence_proxy_async_smem();
               load_v(n_rows - 1);
             } else {
-              atomicOr(&g_status, 1u);
+              expired = true;
             }
           }
+          if (expired) atomicOr(&g_status, 1u);
         }
         __syncwarp();
       } else {
@@ -743,6 +743,9 @@ __global__ void __launch_bounds__(MAXWG * 160, 1) rope_scan_kernel(DecodeArgs a,
           values(n, raise);
         }
       }
+      // a wait that no row barrier has reported (a last row's values, an issuing thread's) ends the CTA
+      // all the same, before its stages are filled again
+      if (expired) sh.fail = 1;
       // ---- the stretch's sums (m, l, (O - c) 2^(10 - kmin)): the second warpgroup's through shared
       //      memory into the first one's, which go to the first slot ----
       const int cr = vr & 15, ct = vr >> 4;
