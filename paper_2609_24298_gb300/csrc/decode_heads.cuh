@@ -242,7 +242,9 @@ __global__ void __launch_bounds__(kHeadThreads, kCombineCtas) combine_kernel(Dec
   if (s0 == 0)
     for (int idx = tid; idx < rv * (kD / 32); idx += kHeadThreads) prefetch_l2(W + 32 * idx);
   const int d0 = 16 * warp + 4 * (lane & 3);  // dims of the back-projection: d0 .. d0 + 3
-  const float4 mu4 = *reinterpret_cast<const float4*>(pool + hv.mu_off + d0);
+  float mu_a[4];  // (a block's means need not be 16-byte aligned)
+#pragma unroll
+  for (int k = 0; k < 4; ++k) mu_a[k] = pool[hv.mu_off + d0 + k];
   // the appends of the next step may start their parameter staging meanwhile
   grid_dep_launch();
   // everything above is independent of the scan; its partials are read only from here on
@@ -398,7 +400,6 @@ __global__ void __launch_bounds__(kHeadThreads, kCombineCtas) combine_kernel(Dec
     }
   }
   // lane share sl holds outputs [sl V / 2, (sl + 1) V / 2) of the 4 V (vector, dim) values
-  const float mu_a[4] = {mu4.x, mu4.y, mu4.z, mu4.w};
 #pragma unroll
   for (int k = 0; k < V / 2; ++k) {
     const int e = sl * (V / 2) + k, v = e >> 2, c = e & 3;

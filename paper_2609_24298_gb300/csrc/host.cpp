@@ -825,6 +825,8 @@ extern "C" cobra_status cobra_params_verify(const void* image, size_t image_byte
     if (e.w_off + (uint64_t)cobra::kD * e.r > hdr.pool_floats || e.mu_off + cobra::kD > hdr.pool_floats ||
         e.wmu_off + (uint64_t)e.r > hdr.pool_floats || (e.cache_off & 255))
       return COBRA_EINVAL;
+    // the kernels read W and W^T mu in 16-byte pieces
+    if (e.r > 0 && ((e.w_off & 3) || (e.wmu_off & 3))) return COBRA_EINVAL;
   }
   return block_checksum(p, image_bytes) == hdr.checksum ? COBRA_OK : COBRA_EINVAL;
 }

@@ -1,6 +1,8 @@
 """GPU parity of cobra_decode_attn (Table alg:kvrobin step 8; App. G) against the oracle's
 plain-definition attention over the same packed codes: max over query heads of
 ||o - o*||_inf / ||o*||_inf <= 2e-3 (bf16 queries, fp32 accumulation)."""
+import struct
+
 import numpy as np
 import pytest
 import torch
@@ -11,6 +13,7 @@ from oracle import rope as orope
 from paper_2609_24298_gb300 import cobra, synth
 
 from .gpu_util import DEV, oracle_decode, oracle_head, oracle_heads_allocated, rel_err, upload
+from .test_lib_params import resign
 
 pytestmark = pytest.mark.gpu
 TOL = 2e-3
@@ -180,3 +183,40 @@ def test_multi_layer_strides():
     params = [oracle_head(s, r, b) for s, (r, b) in zip(srcs, rbs)]
     o, ref, _ = run_decode(params, srcs, 2, 2, 4, [333, 64])
     assert rel_err(o, ref) < TOL
+
+
+@pytest.mark.parametrize("shift", [1, 2, 3])
+def test_mean_at_any_offset_of_the_pool(shift):
+    """An image whose V mean starts off the 16-byte grid verifies, and decodes as one that holds the
+    same mean where the library puts it."""
+    params, srcs = mixed_heads(1, [(32, 2), (64, 3)], cfg=44)
+    r, b = np.array([32, 64], np.int32), np.array([2, 3], np.int32)
+    delta = np.array([p["delta"] for p in params], np.float32)
+    T, G = 300, 4
+    offs, total = cobra.cobra_plan_layout(r, b, 3)
+    W, mu = [p["W"] for p in params], np.stack([p["mu"] for p in params]).astype(np.float32)
+    moved = bytearray(cobra.cobra_params_image(r, b, delta, offs, W, mu.reshape(-1)).tobytes())
+    pool_off, at = struct.unpack_from("<Q", moved, 24)[0], 64 + 64 + 32  # the V head's mu_off
+    mu_off = struct.unpack_from("<Q", moved, at)[0] + shift
+    struct.pack_into("<Q", moved, at, mu_off)
+    mu[1] = np.frombuffer(bytes(moved), np.float32, 128, pool_off + 4 * mu_off)
+    images = [resign(moved), cobra.cobra_params_image(r, b, delta, offs, W, mu.reshape(-1))]
+    g = np.random.default_rng(shift)
+    cache = torch.tensor(g.integers(0, 256, total, dtype=np.uint8), device=DEV)
+    q = torch.tensor(g.standard_normal((1, 1, G, 128)), dtype=torch.bfloat16, device=DEV)
+    desc = cobra.decode_desc(k_head0=0, v_head0=1, layer_stride=1, n_layers=1, n_kv_heads=1, group=G, n_seqs=1,
+                             rows_per_seq=3, q_stride_layer=G * 128, q_stride_seq=G * 128, o_stride_layer=G * 128,
+                             o_stride_seq=G * 128)
+    wsb = cobra.cobra_decode_workspace_size(desc, r, b, [T])
+    ws = torch.empty(wsb, dtype=torch.uint8, device=DEV)
+    info = cobra.cobra_decode_plan(desc, r, b, [T], ws, wsb)
+    lens = torch.tensor([T], dtype=torch.int32, device=DEV)
+    outs = []
+    for img in images:
+        block = torch.empty(img.nbytes, dtype=torch.uint8, device=DEV)
+        cobra.cobra_params_upload(block, img.nbytes, img)
+        out = torch.empty((1, 1, G, 128), dtype=torch.float32, device=DEV)
+        cobra.cobra_decode_attn(block, desc, info, q, cache, lens, None, out, ws, wsb)
+        assert cobra.cobra_check() == cobra.COBRA_OK
+        outs.append(out.cpu())
+    assert torch.equal(outs[0], outs[1]) and torch.isfinite(outs[0]).all()

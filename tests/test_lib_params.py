@@ -129,3 +129,17 @@ def test_inconsistent_head_fields_are_rejected_with_a_valid_checksum(field):
     good = resign(bytearray(img.tobytes()))
     assert cobra.cobra_params_verify(good) == cobra.COBRA_OK  # re-signing alone keeps it valid
     assert cobra.cobra_params_verify(resign(raw)) == cobra.COBRA_EINVAL
+
+
+@pytest.mark.parametrize("field,shift,ok", [("w_off", 1, False), ("w_off", 2, False), ("wmu_off", 1, False),
+                                            ("wmu_off", 2, False), ("w_off", 4, True), ("wmu_off", 4, True),
+                                            ("mu_off", 1, True), ("mu_off", 2, True)])
+def test_offsets_that_the_kernels_cannot_read_are_rejected(field, shift, ok):
+    """W and W^T mu are read in 16-byte pieces: an offset off that grid is rejected on the host, where
+    it would be a misaligned access on the device.  The mean is read by element, at any offset."""
+    raw = bytearray(image()[0].tobytes())
+    at = 64 + 64 * 2 + {"w_off": 24, "mu_off": 32, "wmu_off": 40}[field]  # the head with rank 18
+    off = struct.unpack_from("<Q", raw, at)[0]
+    struct.pack_into("<Q", raw, at, off + shift)
+    want = cobra.COBRA_OK if ok else cobra.COBRA_EINVAL
+    assert cobra.cobra_params_verify(resign(raw)) == want
