@@ -822,8 +822,10 @@ extern "C" cobra_status cobra_params_verify(const void* image, size_t image_byte
     } else if (e.b != 0 || e.delta != 0.0f || e.inv_delta != 0.0f) {
       return COBRA_EINVAL;
     }
-    if (e.w_off + (uint64_t)cobra::kD * e.r > hdr.pool_floats || e.mu_off + cobra::kD > hdr.pool_floats ||
-        e.wmu_off + (uint64_t)e.r > hdr.pool_floats || (e.cache_off & 255))
+    // (no sums: an offset near 2^64 would wrap around)
+    auto outside = [&](uint64_t off, uint64_t n) { return n > hdr.pool_floats || off > hdr.pool_floats - n; };
+    if (outside(e.w_off, (uint64_t)cobra::kD * e.r) || outside(e.mu_off, cobra::kD) || outside(e.wmu_off, e.r) ||
+        (e.cache_off & 255))
       return COBRA_EINVAL;
     // the kernels read W and W^T mu in 16-byte pieces
     if (e.r > 0 && ((e.w_off & 3) || (e.wmu_off & 3))) return COBRA_EINVAL;

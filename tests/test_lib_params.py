@@ -143,3 +143,11 @@ def test_offsets_that_the_kernels_cannot_read_are_rejected(field, shift, ok):
     struct.pack_into("<Q", raw, at, off + shift)
     want = cobra.COBRA_OK if ok else cobra.COBRA_EINVAL
     assert cobra.cobra_params_verify(resign(raw)) == want
+
+
+@pytest.mark.parametrize("field", ["w_off", "mu_off", "wmu_off"])
+def test_offsets_that_wrap_around_are_rejected(field):
+    raw = bytearray(image()[0].tobytes())
+    at = 64 + 64 * 2 + {"w_off": 24, "mu_off": 32, "wmu_off": 40}[field]
+    struct.pack_into("<Q", raw, at, 2 ** 64 - 4)
+    assert cobra.cobra_params_verify(resign(raw)) == cobra.COBRA_EINVAL
