@@ -1,10 +1,9 @@
 """GPU parity of cobra_decode_rope_attn (decode with the rotary embedding applied to the
 rebuilt keys and the query; the paper compresses K before it, Sec. 5 "Scope") against
 oracle.rope over the same packed codes: max over query heads of ||o - o*||_inf / ||o*||_inf
-<= 2e-3, as for the plain decode.  The keys are rebuilt from fp16 hi + lo parts of W_K and
-scored with hi + lo parts of both operands (about 22 bits each), the angles composed from
-fp32 tables of fp64 values (relative error ~1e-7), so the measured error sits far below the
-bound; the cases span every bit width, r = 0 on either side, ragged and empty sequences, the
+<= 2e-3, as for the plain decode.  The keys are rebuilt from fp16 hi + lo parts of W_K (about
+22 bits) with fp32 accumulation and scored in fp32, the angles composed from fp32 tables of fp64
+values (relative error ~1e-7), so the measured error sits far below the bound; the cases span every bit width, r = 0 on either side, ragged and empty sequences, the
 paged layout, groups of 4 and 8, explicit query positions and a position near 32k."""
 import numpy as np
 import pytest
