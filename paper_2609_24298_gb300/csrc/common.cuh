@@ -11,7 +11,7 @@
 namespace cobra {
 
 // ---------------------------------------------------------------------------------------
-// status word: bit 0 = a bounded wait expired
+// status word: bit 0 = a bounded wait expired, bit 1 = an input out of range was skipped or clamped
 // ---------------------------------------------------------------------------------------
 __device__ unsigned int g_status;
 
@@ -25,9 +25,10 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
 // start before the kernel ahead of it in the stream has finished; it calls grid_dep_wait()
 // before reading that kernel's results (a no-op for an ordinary launch).  grid_dep_launch()
 // lets the dependent kernel be scheduled once every CTA of this grid has called it or exited.
-// Every kernel of the library is launched this way and calls grid_dep_wait() on every path
-// before it exits, so that the completion of a kernel implies that of all kernels before it
-// in the stream: a kernel only ever waits for its direct predecessor.
+// A kernel launched this way calls grid_dep_wait() on every path before it exits, so that the
+// completion of a kernel implies that of all kernels before it in the stream: a kernel only ever
+// waits for its direct predecessor.  (Calibration, measured distortion and the static plan are
+// ordinary launches.)
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // pull one 128-byte line into L2 (no register result, nothing to wait for)
@@ -42,9 +43,6 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) {
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_inval(uint32_t bar) {
-  asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void fence_mbar_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -78,18 +76,13 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
+
 // ---------------------------------------------------------------------------------------
 // legacy warp-level MMA (operands in registers) and 8x8 transposition
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                         uint32_t b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                         uint32_t b1) {
-  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
@@ -188,12 +181,6 @@ __host__ __device__ __forceinline__ uint32_t unpack_reg(const uint32_t (&w)[B], 
     const uint32_t hi = w[(wi + 1) < B ? wi + 1 : wi] << (k + nlo);
     return (lo & pair_mask(nlo, k)) | (hi & pair_mask(B - nlo, k + nlo)) | one;
   }
-}
-
-template <int B>
-__host__ __device__ __forceinline__ void unpack_piece(const uint32_t (&w)[B], uint32_t (&o)[16]) {
-#pragma unroll
-  for (int rho = 0; rho < 16; ++rho) o[rho] = unpack_reg<B>(w, rho, kOneH2);
 }
 
 // Words of the piece at p, or zeros when the strip does not exist.

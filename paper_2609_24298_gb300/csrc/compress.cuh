@@ -1,6 +1,7 @@
-// Code-row packing shared by the compress kernels (format v1, see include/cobra.h), and the
-// single-token append (Table alg:kvrobin step 7): y = W^T (x - mu), the fused projection +
-// Hadamard as one multiply (Sec. 3.4), code = clamp(floor(y / Delta + 2^{b-1}), 0, 2^b - 1).
+// The compress kernels' arguments, the projection that the append shares with the query
+// projection, and the single-token append (Table alg:kvrobin step 7): y = W^T (x - mu), the fused
+// projection + Hadamard as one multiply (Sec. 3.4), code = clamp(floor(y / Delta + 2^{b-1}), 0,
+// 2^b - 1), in code rows of format v1 (include/cobra.h).
 //
 // append_kernel    one CTA per (layer, kv head) and run of sequences: projects the new tokens in
 //                  fp32 on CUDA cores and ORs their codes into the rows (other tokens' bits
@@ -26,43 +27,6 @@ struct CompressArgs {
 __device__ __forceinline__ uint32_t pack_bf16(float lo_col, float hi_col) {
   __nv_bfloat162 h = __floats2bfloat162_rn(lo_col, hi_col);
   return *reinterpret_cast<uint32_t*>(&h);
-}
-
-// (token, channel) of code (rho, h) in piece p of strip s.
-__device__ __forceinline__ void piece_code_coords(int side, int s, int p, int rho, int h, int& t, int& i) {
-  const int tau = rho >> 1, u = rho & 1;
-  if (side == 0) {
-    t = 16 * tau + p + 8 * u;
-    i = 2 * s + h;
-  } else {
-    const int c = p >> 2, j = p & 3;
-    t = 16 * tau + 2 * j + 8 * u + h;
-    i = 2 * s + c;
-  }
-}
-
-// Pack one piece (32 codes) from the code tile into B words.
-template <int B>
-__device__ __forceinline__ void pack_piece(const uint8_t* codes, int ldc, int side, int s, int p, uint32_t* dst) {
-  uint32_t w[B];
-#pragma unroll
-  for (int k = 0; k < B; ++k) w[k] = 0u;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-#pragma unroll
-    for (int rho = 0; rho < 16; ++rho) {
-      int t, i;
-      piece_code_coords(side, s, p, rho, h, t, i);
-      const uint32_t c = codes[t * ldc + i];
-#pragma unroll
-      for (int bit = 0; bit < B; ++bit) {
-        const int x = rho * B + bit;
-        w[x >> 4] |= ((c >> bit) & 1u) << (16 * h + (x & 15));
-      }
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < B; ++k) dst[k] = w[k];
 }
 
 // a8: single-token append, and the projection it shares with the query projection (qproj_kernel):
