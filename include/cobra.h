@@ -187,6 +187,11 @@ cobra_status cobra_plan_layout(int n_heads, const int* r, const int* b, long lon
 
 /* ---------------------------------------------------------------------------------------
  * Device parameter block: per-head r, b, Delta, cache offset, fused basis W and mean mu.
+ *
+ * cobra_params_build and cobra_params_upload return with the block in place.  A block (or a plan's
+ * workspace) that a kernel of the caller's writes must not be written by the kernel directly ahead
+ * of cobra_append or a cobra_decode_* call in the stream: these read it while that kernel finishes.
+ * cobra_compress reads it in plain stream order.
  * ------------------------------------------------------------------------------------- */
 
 /* Bytes needed for a parameter block of n_heads heads with ranks r (host [n_heads]). */

@@ -849,14 +849,25 @@ extern "C" cobra_status cobra_params_upload(void* dev_block, size_t block_bytes,
 // goes in large chunks (little per-chunk setup), and the warps that drain the queue finish
 // within one short chunk of one another.  Groups are ordered by code variant (b_K, b_V), then
 // (r_K, r_V), so that the warps working at the same time run the same code.
+//
+// Calls of fewer rows than resident warps, and of kWaveRowsMin to kWaveRowsMax rows per warp, are cut
+// into one wave instead: at most one chunk per warp, of equal estimated cost.  One layer of 8 kv heads
+// at 1 bpd, us per step in one wave against guided chunks: 8 x 8192 tokens (1.7 rows per warp) 32.6 for
+// 36.4, 8 x 32768 (6.7) 55.7 for 57.3, 24 x 8192 (5.1) 45.5 for 55, 24 x 16384 (10.1) 70 for 78.  Between one row
+// and kWaveRowsMin a row more or less is a large part of a warp's share: a ragged batch (24 sequences of
+// 131 to 6001 tokens at 3 bpd, 3 rows per warp) took 51 for 49, so that range stays guided, although
+// sequences of one length gain there as well (8 x 16384: 41 for 43; 1 x 131072: 53 for 81).  Many
+// rows per warp, and wide ones, favour the queue, which evens out what the estimate misses: at 3 bpd
+// 24 x 12288 (7.6) takes 98 for 100, 24 x 16384 (10.1) 122 for 114 and 24 x 24576 (15.2) 169 for 142; at 1 bpd the
+// wave is still ahead at 20 (120 for 131).  kWaveRowsMax lies between.
 // ----------------------------------------------------------------------------------------
 namespace {
 constexpr long long kItemMin = 16 * 1024, kItemMax = 128 * 1024;
-constexpr long long kScanWarps = 152 * 16;  // resident scan warps: 152 SMs x 4 CTAs x 4 warps
+constexpr long long kScanWarps = 152 * 16;  // resident scan warps at most: 152 SMs x 16 (4 query heads, 8 KB rings)
 constexpr long long kGuide = 2;
 constexpr long long kMaxChunks = 32;
 constexpr long long kWaveRowsMin = 5, kWaveRowsMax = 12;
-constexpr long long kWaveMaxChunks = 64;  // per group, when few groups share the warps
+constexpr long long kWaveMaxChunks = 64;  // per group, when few groups share the warps: one round of the combine's weights
 
 // Warp-instructions of the scan per 128-token row pair, in tenths: about 310, and per channel by bit
 // width (measured on the row functions; widths whose codes straddle words cost more).

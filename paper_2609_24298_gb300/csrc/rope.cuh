@@ -34,7 +34,7 @@
 //
 // Bound: the CUDA cores and shared memory, 6 + 3 G instructions per token and two channel pairs (the
 // angles' load, the turn in packed fp32 pairs, per query head one broadcast load and two packed
-// fused multiply-adds).  With 8 warps per SM the latencies between the steps count: X is kept in two
+// fused multiply-adds).  With 8 or 12 warps per SM the latencies between the steps count: X is kept in two
 // halves of 64 columns, so that the next row's MMAs run on the half that has been read while the
 // warps score the other one and accumulate the values.  4 layers x 8 kv heads x 8 x 32768 tokens at
 // 1 bpd: 0.92 to 0.94 ms per call, against 1.80 with the rebuild and the scores on mma.sync (hi + lo of

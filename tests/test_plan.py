@@ -1,8 +1,9 @@
 """CPU tests of the decode work plan (host logic, no device): the chunks of every
 (seq, layer, kv-head) group tile its code rows exactly once, their partial slots are the
 group's consecutive range, the head-group table points back at the right groups, chunks of
-one code variant are taken together in the variants' (b_K, b_V) order, and the chunk sizes
-shrink towards the end of the order without cutting a group into more than 32 chunks."""
+one code variant are taken together in the variants' (b_K, b_V) order.  Large calls' chunks
+shrink towards the end of the order without cutting a group into more than 32; a layer's calls
+are cut into one wave of the resident warps.  A workspace holds the plan of any shorter call."""
 import os
 
 import numpy as np
