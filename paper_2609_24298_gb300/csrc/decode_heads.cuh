@@ -211,16 +211,18 @@ __global__ void __launch_bounds__(kHeadThreads, 2) qproj_kernel(DecodeArgs a, Co
 // One CTA of 256 threads per (layer, kv head) and run of NS sequences.  The kernel is a chain of
 // memory round trips (chunk maxima, chunk sums, the rows of W_V), so every phase spreads its loads
 // over all threads and issues them together; a head's W_V is read again for each run (from L2).
-// Against one CTA per head and run of 16 query vectors, a step over 1 layer x 8 kv heads takes
-// 23 us for 25.9 (1 x 2048 tokens), 50 for 67 (24 ragged sequences at 3 bpd) and 63 for 80
-// (8 x 32768).  NS = 1 spreads a call over the most CTAs; with 4 query heads, calls that would take
-// more than two rounds of resident CTAs share W_V between two sequences where that takes fewer rounds
-// (combine_seqs): 32 layers x 8 heads x 16 sequences 33.5 us for 46.5 with NS = 1, x 64 sequences 125 for
-// 187 (112 with runs of 16 vectors); 1 layer x 64 sequences would take 8.6 for 8.5, its step 45.7 for 44.2.
+// Two forms (combine_many), us alone, against 20, 33.5 and 112 with one CTA per head and run of 16
+// query vectors, for 32 layers x 8 heads of 4 query heads and 8, 16 and 64 sequences:
+//   kCombineFew   one sequence, 3 CTAs per SM, eight loads in flight per thread: the most CTAs for a
+//                 call, 24, 47 and 185.  A step over 1 layer x 8 kv heads takes 23 us for 25.9 (1 x 2048
+//                 tokens), 50 for 67 (24 ragged sequences at 3 bpd) and 63 for 80 (8 x 32768).
+//   kCombineMany  runs of 8 query vectors, 4 CTAs per SM, four loads in flight: the most sequences at a
+//                 time, 18, 31 and 111.
 // ---------------------------------------------------------------------------------------
-constexpr int kCombineCtas = 3;  // resident per SM
-template <int G, int NS>
-__global__ void __launch_bounds__(kHeadThreads, kCombineCtas) combine_kernel(DecodeArgs a) {
+constexpr int kCombineFew = 3, kCombineMany = 4;  // resident CTAs per SM
+template <int G, int NS, int CTAS>
+__global__ void __launch_bounds__(kHeadThreads, CTAS) combine_kernel(DecodeArgs a) {
+  constexpr int UB = CTAS == kCombineMany ? 4 : 8;  // loads in flight per thread
   constexpr int V = G * NS;  // query vectors of the CTA: vector v = query head v % G of sequence s0 + v / G
   static_assert(V <= kHeadThreads / 32, "a warp per vector");
   __shared__ float wts[V][kWtChunk];          // weights 2^(m_k - m*) / l* of a round of chunks
@@ -242,9 +244,15 @@ __global__ void __launch_bounds__(kHeadThreads, kCombineCtas) combine_kernel(Dec
   if (s0 == 0)
     for (int idx = tid; idx < rv * (kD / 32); idx += kHeadThreads) prefetch_l2(W + 32 * idx);
   const int d0 = 16 * warp + 4 * (lane & 3);  // dims of the back-projection: d0 .. d0 + 3
-  float mu_a[4];  // (a block's means need not be 16-byte aligned)
+  float mu_a[4];
+  const float* mu = pool + hv.mu_off + d0;
+  if (hv.mu_off % 4 == 0) {
+    const float4 m4 = *reinterpret_cast<const float4*>(mu);
+    mu_a[0] = m4.x, mu_a[1] = m4.y, mu_a[2] = m4.z, mu_a[3] = m4.w;
+  } else {  // (another tool's block)
 #pragma unroll
-  for (int k = 0; k < 4; ++k) mu_a[k] = pool[hv.mu_off + d0 + k];
+    for (int k = 0; k < 4; ++k) mu_a[k] = mu[k];
+  }
   // the appends of the next step may start their parameter staging meanwhile
   grid_dep_launch();
   // everything above is independent of the scan; its partials are read only from here on
@@ -293,8 +301,8 @@ __global__ void __launch_bounds__(kHeadThreads, kCombineCtas) combine_kernel(Dec
   }
   __syncthreads();
   // (2) weighted chunk sums: thread (channel quad cq, vector v, chunk share p) of rw = r_V
-  //     rounded up to 32, 64 or 128 channels sums 16-byte entries of chunks p, p + np, ..., eight
-  //     loads in flight; the shares are added through shared memory.
+  //     rounded up to 32, 64 or 128 channels sums 16-byte entries of chunks p, p + np, ..., UB loads
+  //     in flight; the shares are added through shared memory.
   const int rw = rv <= 32 ? 32 : rv <= 64 ? 64 : kD;
   const int nq = rw / 4, np = kHeadThreads / (nq * V);  // np >= 1 (V = 8, rw = 128)
   {
@@ -318,18 +326,18 @@ __global__ void __launch_bounds__(kHeadThreads, kCombineCtas) combine_kernel(Dec
       // the partial's channels start 4 floats in and every stride is a multiple of 4 floats
       const float4* px = reinterpret_cast<const float4*>(first(v) + (size_t)k0 * pstride + 4 + 4 * cq);
       const int kr = min(kWtChunk, n - k0);
-      for (int kb = p; kb < kr; kb += 8 * np) {
-        float4 x[8];
-        float w[8];
+      for (int kb = p; kb < kr; kb += UB * np) {
+        float4 x[UB];
+        float w[UB];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
+        for (int u = 0; u < UB; ++u) {
           const int k = kb + u * np;
           w[u] = k < kr ? wts[v][k] : 0.f;
           // an empty chunk's value entries were never written
           x[u] = w[u] != 0.f ? px[(size_t)k * (pstride / 4)] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
+        for (int u = 0; u < UB; ++u) {
           acc.x += w[u] * x[u].x;
           acc.y += w[u] * x[u].y;
           acc.z += w[u] * x[u].z;
@@ -360,7 +368,7 @@ __global__ void __launch_bounds__(kHeadThreads, kCombineCtas) combine_kernel(Dec
     }
   }
   __syncthreads();
-  // (3) o = mu_V + W_V zbar: a warp has 16 dims, its lanes 4 dims x every eighth row of W_V (eight
+  // (3) o = mu_V + W_V zbar: a warp has 16 dims, its lanes 4 dims x every eighth row of W_V (UB
   //     16-byte loads in flight); the eight row shares are added by halving exchanges, after which
   //     a lane holds V / 2 consecutive outputs.
   float o[4 * V];
@@ -368,13 +376,13 @@ __global__ void __launch_bounds__(kHeadThreads, kCombineCtas) combine_kernel(Dec
   for (int k = 0; k < 4 * V; ++k) o[k] = 0.f;
   const int sl = lane >> 2;
   const float4* W4 = reinterpret_cast<const float4*>(W + d0);
-  for (int i0 = sl; i0 < rv; i0 += 64) {
-    float4 w[8];
+  for (int i0 = sl; i0 < rv; i0 += 8 * UB) {
+    float4 w[UB];
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
+    for (int u = 0; u < UB; ++u)
       w[u] = i0 + 8 * u < rv ? __ldg(W4 + (i0 + 8 * u) * (kD / 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < UB; ++u) {
       // rows past r_V have w = 0; their zbar is finite (zeros, or within rw <= 128 rows)
       const float* zr = red + (i0 + 8 * u < rv ? i0 + 8 * u : 0) * V;
 #pragma unroll
@@ -405,9 +413,9 @@ __global__ void __launch_bounds__(kHeadThreads, kCombineCtas) combine_kernel(Dec
     const int e = sl * (V / 2) + k, v = e >> 2, c = e & 3;
     const WsGroup& gr = NS == 1 || v < G ? g0 : g1;
     if (NS > 1 && v >= G && s0 + 1 >= S) break;
-    const float mu = (V == 8) ? mu_a[k & 3] : ((sl & 1) ? mu_a[2 + k] : mu_a[k]);
+    const float muk = (V == 8) ? mu_a[k & 3] : ((sl & 1) ? mu_a[2 + k] : mu_a[k]);
     // the output is only 4-byte aligned in general
-    a.out[gr.layer * a.o_sl + gr.seq * a.o_ss + (long long)(gr.kv * G + v % G) * kD + d0 + c] = chunks(v) > 0 ? mu + o[k] : 0.f;
+    a.out[gr.layer * a.o_sl + gr.seq * a.o_ss + (long long)(gr.kv * G + v % G) * kD + d0 + c] = chunks(v) > 0 ? muk + o[k] : 0.f;
   }
 }
 

@@ -231,13 +231,14 @@ ProjSplit proj_split(long long heads, int n_seqs) {
   return {(n_seqs + spb - 1) / spb, spb};
 }
 
-// Sequences per combine CTA: two where that is fewer rounds of resident CTAs, by more than a CTA of
-// two sequences takes longer (5.1 against 6.5 us per round), and the call has more than two rounds
-// (kernels of one or two rounds hide behind the scan's tail; NS = 1 starts sooner).
-int combine_seqs(int group, long long n_heads, int n_seqs) {
-  const long long resident = (long long)kCombineCtas * sm_count();
-  auto rounds = [&](int ns) { return (n_heads * ((n_seqs + ns - 1) / ns) + resident - 1) / resident; };
-  return group == 4 && rounds(1) > 2 && 3 * rounds(1) > 4 * rounds(2) ? 2 : 1;
+// Whether a call's combine runs in the form for many groups: past two rounds of the other form's
+// resident CTAs (calls of one or two rounds hide behind the scan's tail), where the rounds saved
+// outweigh their length (4 query heads: 7.8 us for two sequences against 5.1 for one; 8: 8.0 against 6.6).
+bool combine_many(int group, long long n_heads, int n_seqs) {
+  const long long sms = sm_count();
+  auto rounds = [&](int ns, int ctas) { return (n_heads * ((n_seqs + ns - 1) / ns) + ctas * sms - 1) / (ctas * sms); };
+  const long long few = rounds(1, kCombineFew), many = rounds(8 / group, kCombineMany);
+  return few > 2 && (group == 4 ? 2 * few > 3 * many : 5 * few > 6 * many);
 }
 
 // validated append arguments for one side
@@ -326,11 +327,12 @@ cobra_status launch_decode(const DecodeArgs& a, int n_heads, int n_seqs, int n_i
   }
   if (stages & kCombine) {
     // its prologue (the plan, the L2 prefetch of W_V) overlaps the scan's tail
-    const int ns = combine_seqs(G, n_heads, n_seqs);
+    const bool many = combine_many(G, n_heads, n_seqs);
+    const int ns = many ? 8 / G : 1;
     const long long grid = (long long)n_heads * ((n_seqs + ns - 1) / ns);
     if (grid > 0x7fffffffLL) return COBRA_EINVAL;
-    if (launch_pdl(ns == 2 ? combine_kernel<G, 8 / G> : combine_kernel<G, 1>, (unsigned)grid, kHeadThreads, 0, s, a) !=
-        cudaSuccess)
+    if (launch_pdl(many ? combine_kernel<G, 8 / G, kCombineMany> : combine_kernel<G, 1, kCombineFew>, (unsigned)grid,
+                   kHeadThreads, 0, s, a) != cudaSuccess)
       return COBRA_ECUDA;
   }
   return COBRA_OK;
