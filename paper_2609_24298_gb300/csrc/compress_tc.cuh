@@ -472,17 +472,35 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // Basis row of channel ch as nsplit bf16 terms, the A operand of the MMAs: TMEM lane ch,
     // column kTcWCol + 64 sp + c holds dims 2c (low half) and 2c + 1 of term sp; rows of
     // channels >= r are zero.
+    // The warp reads its 32 rows together, 16 bytes per lane and two half rows at a time, and turns
+    // them through its share of the row staging (16-byte pieces, swizzled by row): a lane reading its
+    // own row touches 32 lines per load, which a short call waits for (K and V of a 2001-token chunk 14.4
+    // against 16.9 us).
     {
-      const float4* wrow = reinterpret_cast<const float4*>(pool + he.w_off + (size_t)(ch < r ? ch : 0) * kD);
-      float4 wv[32];  // the whole row in flight at once
+      const int c0 = 32 * (warp & 3);
+      const float4* wq = reinterpret_cast<const float4*>(pool + he.w_off) + (size_t)(c0 + (lane >> 4)) * (kD / 4) + (lane & 15);
+      float4 wv[2][16];  // [half][row pair], all in flight at once
 #pragma unroll
-      for (int u = 0; u < 32; ++u) wv[u] = ch < r ? wrow[u] : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int u = 0; u < 16; ++u)
+          wv[h][u] = c0 + 2 * u + (lane >> 4) < r ? wq[u * (2 * kD / 4) + 16 * h] : make_float4(0.f, 0.f, 0.f, 0.f);
+      float4* turn = reinterpret_cast<float4*>(rsm) + (warp & 3) * (2 * kTcRowStage / 4 / 16);  // [row][16 pieces]
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
+        if ((q & 1) == 0) {
+          __syncwarp();  // the other half has been read
+#pragma unroll
+          for (int u = 0; u < 16; ++u) {
+            const int row = 2 * u + (lane >> 4);
+            turn[16 * row + ((lane & 15) ^ (row & 15))] = wv[q >> 1][u];
+          }
+          __syncwarp();
+        }
         float rem[32];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          const float4 f = wv[8 * q + u];
+          const float4 f = turn[16 * lane + ((8 * (q & 1) + u) ^ (lane & 15))];
           rem[4 * u] = f.x;
           rem[4 * u + 1] = f.y;
           rem[4 * u + 2] = f.z;
