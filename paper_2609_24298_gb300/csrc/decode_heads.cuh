@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kHeadThreads, 2) qproj_kernel(DecodeArgs a, Co
 //                 call, 24, 47 and 185.  A step over 1 layer x 8 kv heads takes 23 us for 25.9 (1 x 2048
 //                 tokens), 50 for 67 (24 ragged sequences at 3 bpd) and 63 for 80 (8 x 32768).
 //   kCombineMany  runs of 8 query vectors, 4 CTAs per SM, four loads in flight: the most sequences at a
-//                 time, 18, 31 and 111.
+//                 time, 17, 30 and 108.
 // ---------------------------------------------------------------------------------------
 constexpr int kCombineFew = 3, kCombineMany = 4;  // resident CTAs per SM
 template <int G, int NS, int CTAS>
@@ -407,15 +407,28 @@ __global__ void __launch_bounds__(kHeadThreads, CTAS) combine_kernel(DecodeArgs 
       }
     }
   }
-  // lane share sl holds outputs [sl V / 2, (sl + 1) V / 2) of the 4 V (vector, dim) values
+  // lane share sl holds outputs [sl V / 2, (sl + 1) V / 2) of the 4 V (vector, dim) values: 2 or 4
+  // consecutive dims c0 .. of vector v, which leave in one store where the output's rows are aligned
+  // (it may be host memory, where every store costs: a step that writes 4 MB there by element took
+  // 0.84 ms for 0.77)
+  const int v = sl * (V / 2) >> 2, c0 = sl * (V / 2) & 3;
+  const WsGroup& gr = NS == 1 || v < G ? g0 : g1;
+  if (NS > 1 && v >= G && s0 + 1 >= S) return;
+  float* dst = a.out + gr.layer * a.o_sl + gr.seq * a.o_ss + (long long)(gr.kv * G + v % G) * kD + d0 + c0;
+  const bool wide = ((reinterpret_cast<uintptr_t>(a.out) | (uintptr_t)(4 * a.o_sl) | (uintptr_t)(4 * a.o_ss)) & 15) == 0;
+  float res[V / 2];
 #pragma unroll
   for (int k = 0; k < V / 2; ++k) {
-    const int e = sl * (V / 2) + k, v = e >> 2, c = e & 3;
-    const WsGroup& gr = NS == 1 || v < G ? g0 : g1;
-    if (NS > 1 && v >= G && s0 + 1 >= S) break;
     const float muk = (V == 8) ? mu_a[k & 3] : ((sl & 1) ? mu_a[2 + k] : mu_a[k]);
-    // the output is only 4-byte aligned in general
-    a.out[gr.layer * a.o_sl + gr.seq * a.o_ss + (long long)(gr.kv * G + v % G) * kD + d0 + c] = chunks(v) > 0 ? muk + o[k] : 0.f;
+    res[k] = chunks(v) > 0 ? muk + o[k] : 0.f;
+  }
+  if (!wide) {  // 4-byte aligned in general
+#pragma unroll
+    for (int k = 0; k < V / 2; ++k) dst[k] = res[k];
+  } else if constexpr (V == 8) {
+    *reinterpret_cast<float4*>(dst) = make_float4(res[0], res[1], res[2], res[3]);
+  } else {
+    *reinterpret_cast<float2*>(dst) = make_float2(res[0], res[1]);
   }
 }
 

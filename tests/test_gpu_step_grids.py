@@ -29,9 +29,9 @@ def heads():
 
 def step(heads, layers, S, G, layer=None, shift=0, paged=False, cap=500, empty=None):
     """One step over `layers` copies of the two heads (or over layer `layer` alone) on a cache of
-    constant bytes; inputs are the same whatever the form.  shift: elements the inputs are moved
-    from their 16-byte boundary; paged: the sequences' pages in random order; empty: a sequence
-    whose length reads 0 in the attention."""
+    constant bytes; inputs are the same whatever the form.  shift: elements the inputs and outputs
+    are moved from their 16-byte boundary; paged: the sequences' pages in random order; empty: a
+    sequence whose length reads 0 in the attention."""
     n = 2 * layers
     params = heads[:2] * layers + heads[2:] * layers
     n_slots = S * ROWS
@@ -63,7 +63,8 @@ def step(heads, layers, S, G, layer=None, shift=0, paged=False, cap=500, empty=N
     wsb = cobra.cobra_decode_workspace_size(desc, r, b, lens)
     ws = torch.empty(wsb, dtype=torch.uint8, device=DEV)
     info = cobra.cobra_decode_plan(desc, r, b, lens, ws, wsb)
-    out = torch.full((L, S, 2 * G, 128), float("nan"), dtype=torch.float32, device=DEV)
+    obuf = torch.full((L * S * 2 * G * 128 + 4,), float("nan"), dtype=torch.float32, device=DEV)
+    out = obuf[shift % 4:shift % 4 + obuf.numel() - 4].view(L, S, 2 * G, 128)
     ld, pos = torch.tensor(lens, device=DEV), torch.tensor(lens - 1, device=DEV)
     if empty is not None:
         ld[empty] = 0
@@ -76,7 +77,7 @@ def step(heads, layers, S, G, layer=None, shift=0, paged=False, cap=500, empty=N
 @pytest.mark.parametrize("S,paged", [(1, False), (3, True), (41, False), (41, True), (83, False)])
 def test_alignment_of_tokens_and_queries(heads, S, G, paged):
     c0, o0, *_ = step(heads, 1, S, G, paged=paged)
-    for shift in (1, 4):
+    for shift in (1, 2, 4):
         c1, o1, *_ = step(heads, 1, S, G, shift=shift, paged=paged)
         assert np.array_equal(c0, c1) and np.array_equal(o0, o1)
     if paged:  # the same rows wherever their pages lie
@@ -108,5 +109,6 @@ def test_combine_of_two_sequences_per_cta(heads, S, empty):
     for layer in (0, 37, 79):
         _, o1, *_ = step(heads, layers, S, 4, layer=layer, cap=128, empty=empty)
         assert np.array_equal(o1[0], o0[layer])
+    assert np.array_equal(o0, step(heads, layers, S, 4, cap=128, empty=empty, shift=1)[1])
     if empty is not None:
         assert np.all(o0[:, empty] == 0) and np.all(o0[:, empty + 1] != 0)
