@@ -67,8 +67,8 @@ struct Heads {
 //    of work covers a copy and the ring is no larger than a pair.  (One lane issuing bulk copies on
 //    an mbarrier per stage took 130 warp-instructions per row pair of about 1100.  Two stages of
 //    whole pairs left 6 warps per SM at 4 bpd and single-buffered rows at 3: 539 against 453 us per
-//    step for 2 layers x 32 ragged sequences at 4 bpd, 817 against 795 for 32 layers x 8 x 32768
-//    tokens at 1 bpd.);
+//    step for one draw of 2 layers x 32 ragged sequences at 4 bpd, 817 against 795 for 32 layers x 8 x
+//    32768 tokens at 1 bpd.);
 //  * scores s_t (log2 units) come from the K codes by f16 MMA; probabilities are taken
 //    against a reference max that is raised (and the accumulators rescaled) only when a
 //    row's max exceeds it by more than kTau, so most rows need no rescale;
