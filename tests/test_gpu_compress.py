@@ -245,3 +245,14 @@ def test_parameters_written_by_the_kernel_ahead():
         assert torch.equal(cache, again)
         got.append(cache)
     assert torch.equal(got[0], got[2]) and not torch.equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("side", [0, 1])
+@pytest.mark.parametrize("T", [1, 300, 2001])
+def test_heads_without_codes_among_others(side, T):
+    """A head of rank 0 has no rows; its CTAs leave without work beside those of the other heads."""
+    srcs = [synth.HeadSource(12, 0, h, side, (0.3, 2.5)) for h in range(4)]
+    params = [oracle_head(s, r, b) for s, (r, b) in zip(srcs, [(0, 1), (64, 2), (0, 1), (18, 6)])]
+    host, offs, r, b, xs = run_compress(params, srcs, T, side)
+    for h in (1, 3):
+        check_head(host, offs[h], side, params[h], xs[0][:, h], T)
